@@ -92,13 +92,13 @@ extern "C" {
                                      else gather */
 #define STARMAP_KERNEL_GATHER  1  /* one thread per point, CSR loop over moments */
 #define STARMAP_KERNEL_TILED   2  /* TMA-staged tiles, moments streamed by order (FP32, 2D P_N,
-                                     N <= 63); tile height chosen by N, and 5-row tiles at
-                                     one CTA per SM where the tables of the 10-row tiles
-                                     leave no room for their ring (N >= 56 or so); up to
-                                     2^36 values per staggered grid */
-#define STARMAP_KERNEL_TILED_TALL  3  /* tiled, 64 x 10 tiles, one CTA per SM (E_UNSUPPORTED where
-                                         their tables do not fit, N >= 56 or so) */
-#define STARMAP_KERNEL_TILED_SHORT 4  /* tiled, 64 x 5 tiles, two CTAs per SM */
+                                     N <= 63); 10-row tiles, but 5-row ones on a grid too
+                                     small to give half the SMs a tile and where the tables
+                                     of the 10-row tiles leave no room for their ring
+                                     (N >= 56); up to 2^36 values per staggered grid */
+#define STARMAP_KERNEL_TILED_TALL  3  /* tiled, 64 x 10 tiles (E_UNSUPPORTED where their
+                                         tables do not fit, N >= 56) */
+#define STARMAP_KERNEL_TILED_SHORT 4  /* tiled, 64 x 5 tiles */
 
 /* Closure of the moment hierarchy.  NONE: the P_N truncation of section 3
  * (moments of order N+1 are zero).  MLP8: not in the paper (its outlook,
@@ -322,7 +322,7 @@ int starmap_health_verdict(double l2_start, double l2_end, double t_span, double
  * odd halves).  Time and step count are not advanced.  For profiling and for
  * callers composing their own schedule of eq. solution_operator_full_step.
  * With the fused schedule, parity 2 (which = 1) runs two fused inner steps
- * E_dt O_dt E_dt O_dt (two launches and their boundary refreshes). */
+ * E_dt O_dt E_dt O_dt (two launches, each with a refresh of the odd boundary copies). */
 int starmap_pass(starmap_t* h, int parity, int which);
 /* Step until t_out lies in (t, t + dt] and keep the solution of the last
  * two time levels; starmap_output() then returns the linear interpolation
@@ -535,9 +535,9 @@ int starmap_mlp_shuffle(starmap_mlp_t* net, const int32_t* index, size_t count, 
  * one CUDA graph launch: per pass, one persistent kernel walks the tiles of
  * all instances with each instance's own tables (work units of all
  * instances dealt to the CTAs by load: strips of consecutive tiles in y
- * for short tiles, single tiles for long ones), then one kernel refreshes
- * the boundary copies of every instance; the pass sequence of a step count
- * is captured once and replayed.  The
+ * for short tiles, single tiles for long ones), which also writes the
+ * boundary copies; the pass sequence of a step count is captured once and
+ * replayed.  The
  * schedule is cfgs[0].schedule for all; cfgs[0].cuda_stream (if not NULL)
  * must be a non-default stream (graphs are captured on it).  Tile shape:
  * cfgs[0].kernel = STARMAP_KERNEL_TILED_TALL or _TILED_SHORT forces 64 x 10

@@ -42,6 +42,7 @@ struct starmap_s {
     long steps = 0;
     int p[2] = {1, 1};
     int nxg[4] = {0, 0, 0, 0}, nyg[4] = {0, 0, 0, 0}, Kg[4] = {0, 0, 0, 0};
+    int cpg[4] = {0, 0, 0, 0};            // row pitch of a grid's coefficients and sources on the device
     long pitch = 0, rows = 0;
     std::vector<int> members[4];          // component ids per grid, by local index
     size_t esize = 8;
@@ -110,6 +111,7 @@ struct starmap_batch_s {
     bool own_stream = false;
     int schedule = STARMAP_SCHEDULE_MERGED;
     int variant = 1;                       // tile height of every instance (see starmap_batch_create)
+    int shape = 0;                         // the batch kernel (tiled_batch_shape)
     double tuned_ms[2] = {-1.0, -1.0};     // autotuner: ms per step with 10-row / 5-row tiles (-1: not timed)
     int strip = 192;                       // stages per strip of short tiles (batch_plan)
     bool from_cache = false;               // the tuning came from the cache file
@@ -121,8 +123,6 @@ struct starmap_batch_s {
     void* dev_params = nullptr;
     void* dev_items = nullptr;             // per CTA: strided runs (instance, first tile, count, stride)
     int* dev_off = nullptr;                // CTA b's runs: items[off[b]] .. items[off[b + 1] - 1]
-    GhostJob* dev_ghosts[2] = {nullptr, nullptr};   // boundary refresh after even / odd passes
-    int nghosts[2] = {0, 0};
     int smem = 0;
     int grid = 0;
     std::vector<std::pair<long, cudaGraphExec_t>> graphs;   // captured step sequences by step count
@@ -171,6 +171,7 @@ GridDev<T> grid_dev(const starmap_t* h, int g) {
     d.ny = h->nyg[g];
     d.K = h->Kg[g];
     d.coef = (T*)h->coef[g];
+    d.cp = h->cpg[g];
     return d;
 }
 
@@ -249,23 +250,27 @@ int rebuild_tables(starmap_t* h) {
 // Stored as a = exp(-c dt/2), b = dt/2 E(-c dt/2), A = exp(-c dt), B = dt E(-c dt).
 template <class T>
 int upload_coefficients(starmap_t* h, int g) {
-    const long plane = (long)h->nxg[g] * h->nyg[g];
+    const long plane = (long)h->cpg[g] * h->nyg[g];     // rows padded to cpg (the padding is never used)
     if (plane == 0) return STARMAP_OK;
     std::vector<T> buf((size_t)h->nclasses * 4 * plane);
     const std::vector<double>& sa = h->sig_a[g];
     const std::vector<double>& ss = h->sig_s[g];
     const double dt = h->dt;
+    const int nx = h->nxg[g], ny = h->nyg[g];
     for (int cls = 0; cls < h->nclasses; ++cls) {
-        for (long i = 0; i < plane; ++i) {
-            double c;
-            if (cls == 0) c = sa[i];
-            else if (h->sl_factor.empty()) c = sa[i] + ss[i];
-            else c = sa[i] + ss[i] - ss[i] * h->sl_factor[cls];
-            T* dst = buf.data() + (size_t)cls * 4 * plane + i;
-            dst[0] = (T)std::exp(-c * dt / 2);
-            dst[plane] = (T)(dt / 2 * expm1div(-c * dt / 2));
-            dst[2 * plane] = (T)std::exp(-c * dt);
-            dst[3 * plane] = (T)(dt * expm1div(-c * dt));
+        for (int y = 0; y < ny; ++y) {
+            T* dst = buf.data() + (size_t)cls * 4 * plane + (size_t)y * h->cpg[g];
+            for (int x = 0; x < nx; ++x, ++dst) {
+                const size_t i = (size_t)y * nx + x;
+                double c;
+                if (cls == 0) c = sa[i];
+                else if (h->sl_factor.empty()) c = sa[i] + ss[i];
+                else c = sa[i] + ss[i] - ss[i] * h->sl_factor[cls];
+                dst[0] = (T)std::exp(-c * dt / 2);
+                dst[plane] = (T)(dt / 2 * expm1div(-c * dt / 2));
+                dst[2 * plane] = (T)std::exp(-c * dt);
+                dst[3 * plane] = (T)(dt * expm1div(-c * dt));
+            }
         }
     }
     CK(cudaMemcpyAsync(h->coef[g], buf.data(), buf.size() * sizeof(T), cudaMemcpyHostToDevice, h->stream), "upload coefficients");
@@ -277,7 +282,7 @@ int ensure_coef_alloc(starmap_t* h) {
     if (h->ncls_alloc >= h->nclasses) return STARMAP_OK;
     for (int g = 0; g < 4; ++g) {
         if (h->coef[g]) { cudaFree(h->coef[g]); h->coef[g] = nullptr; }
-        size_t bytes = std::max<size_t>(1, (size_t)h->nclasses * 4 * h->nxg[g] * h->nyg[g]) * h->esize;
+        size_t bytes = std::max<size_t>(1, (size_t)h->nclasses * 4 * h->cpg[g] * h->nyg[g]) * h->esize;
         CK(dev_alloc(&h->coef[g], bytes), "cudaMalloc coefficients");
     }
     h->ncls_alloc = h->nclasses;
@@ -318,16 +323,6 @@ int run_pass(starmap_t* h, bool odd, int which) {
     if (h->kernel_used != STARMAP_KERNEL_GATHER) {
         int rc = tiled_pass(h->tiled, odd, which, h->stream);
         if (rc) return fail(h, rc, tiled_error(h->tiled));
-        // the tiled pass leaves the boundary copies to this refresh (scattered
-        // single-value stores would otherwise gate the boundary tiles)
-        GhostPassArgs<T> ga;
-        const int go[2] = {odd ? 1 : 0, odd ? 2 : 3};
-        for (int q = 0; q < 2; ++q) { ga.g[q] = grid_dev<T>(h, go[q]); ga.grid[q] = go[q]; }
-        ga.pitch = h->pitch;
-        ga.p[0] = h->p[0];
-        ga.p[1] = h->p[1];
-        if (launch_fill_ghosts_pass<T>(ga, h->stream, tiled_overlap(h->tiled, odd)))
-            return cuda_fail(h, cudaGetLastError(), "ghost refresh");
         return STARMAP_OK;
     }
     const int gl[2] = {odd ? 1 : 0, odd ? 2 : 3};
@@ -659,7 +654,8 @@ int starmap_host_expm1div(double* c, size_t count) {
     return STARMAP_OK;
 }
 
-int starmap_create(const starmap_config* cfg, starmap_t** out) {
+// starmap_create; shape: see TiledGeometry.
+static int create_handle(const starmap_config* cfg, int shape, starmap_t** out) {
     if (!out) return fail(nullptr, STARMAP_E_ARG, "out is NULL");
     *out = nullptr;
     if (!cfg) return fail(nullptr, STARMAP_E_ARG, "cfg is NULL");
@@ -722,6 +718,7 @@ int starmap_create(const starmap_config* cfg, starmap_t** out) {
         h->nxg[g] = xnode ? c.n[0] + 1 - h->p[0] : c.n[0];
         h->nyg[g] = ynode ? c.n[1] + 1 - h->p[1] : c.n[1];
         h->Kg[g] = h->sys.grid_count[g];
+        h->cpg[g] = (h->nxg[g] + 31) / 32 * 32;
     }
     for (int j = 0; j < h->ncomp; ++j) h->members[h->sys.moms[j].grid].push_back(j);
     for (int g = 0; g < 4; ++g)
@@ -749,7 +746,7 @@ int starmap_create(const starmap_config* cfg, starmap_t** out) {
         delete h;
         return fail(nullptr, STARMAP_E_UNSUPPORTED, "tiled kernel needs FP32, the 2D P_N system, N <= 63 and TMA support");
     }
-    int variant = tiled_default_variant(h->nsys);
+    int variant = tiled_default_variant(h->nsys, nxmax, nymax);
     if (c.kernel == STARMAP_KERNEL_TILED_TALL) variant = 0;
     if (c.kernel == STARMAP_KERNEL_TILED_SHORT) variant = 1;
     h->kernel_used = (want_tiled || (c.kernel == STARMAP_KERNEL_AUTO && tiled_ok))
@@ -783,9 +780,9 @@ int starmap_create(const starmap_config* cfg, starmap_t** out) {
         TiledGeometry geo;
         for (int g = 0; g < 4; ++g) {
             geo.base[g] = h->base[g]; geo.cstride[g] = h->cstride[g];
-            geo.nx[g] = h->nxg[g]; geo.ny[g] = h->nyg[g]; geo.K[g] = h->Kg[g];
+            geo.nx[g] = h->nxg[g]; geo.ny[g] = h->nyg[g]; geo.K[g] = h->Kg[g]; geo.cp[g] = h->cpg[g];
         }
-        geo.pitch = h->pitch; geo.rows = h->rows; geo.p[0] = h->p[0]; geo.p[1] = h->p[1]; geo.N = h->nsys;
+        geo.pitch = h->pitch; geo.rows = h->rows; geo.p[0] = h->p[0]; geo.p[1] = h->p[1]; geo.N = h->nsys; geo.shape = shape;
         geo.variant = h->kernel_used == STARMAP_KERNEL_TILED_SHORT ? 1 : 0;
         int rc = tiled_create(geo, &h->tiled);
         if (rc) { std::string m = h->tiled ? tiled_error(h->tiled) : "tiled kernel setup failed"; return bail(fail(h, rc, m)); }
@@ -805,9 +802,9 @@ int starmap_create(const starmap_config* cfg, starmap_t** out) {
         TiledGeometry geo;
         for (int g = 0; g < 4; ++g) {
             geo.base[g] = h->base[g]; geo.cstride[g] = h->cstride[g];
-            geo.nx[g] = h->nxg[g]; geo.ny[g] = h->nyg[g]; geo.K[g] = h->Kg[g];
+            geo.nx[g] = h->nxg[g]; geo.ny[g] = h->nyg[g]; geo.K[g] = h->Kg[g]; geo.cp[g] = h->cpg[g];
         }
-        geo.pitch = h->pitch; geo.rows = h->rows; geo.p[0] = h->p[0]; geo.p[1] = h->p[1]; geo.N = h->nsys;
+        geo.pitch = h->pitch; geo.rows = h->rows; geo.p[0] = h->p[0]; geo.p[1] = h->p[1]; geo.N = h->nsys; geo.shape = shape;
         geo.variant = 1;
         rc = tiled_create(geo, &h->tiled);
         if (rc) return bail(fail(h, rc, h->tiled ? tiled_error(h->tiled) : "tiled kernel setup failed"));
@@ -843,6 +840,8 @@ int starmap_create(const starmap_config* cfg, starmap_t** out) {
     *out = h;
     return STARMAP_OK;
 }
+
+int starmap_create(const starmap_config* cfg, starmap_t** out) { return create_handle(cfg, -1, out); }
 
 void starmap_destroy(starmap_t* h) {
     if (!h) return;
@@ -938,6 +937,7 @@ int starmap_set_source(starmap_t* h, int j, const double* q, size_t count) {
     if (h->frozen[j] && q) return fail(h, STARMAP_E_ARG, "the order-8 components of the closure take no source");
     CK(cudaStreamSynchronize(h->stream), "set_source");
     size_t np = comp_points(h, j);
+    const int g = h->sys.moms[j].grid;
     if (!q) {
         if (j < (int)h->src_sq.size()) h->src_sq[j] = 0.0;
         if (h->src_slot[j] >= 0) {
@@ -959,7 +959,7 @@ int starmap_set_source(starmap_t* h, int j, const double* q, size_t count) {
     const bool new_slot = h->src_slot[j] < 0;
     if (new_slot) {
         void* d = nullptr;
-        CK(dev_alloc(&d, np * h->esize), "cudaMalloc source");
+        CK(dev_alloc(&d, (size_t)h->cpg[g] * h->nyg[g] * h->esize), "cudaMalloc source");
         h->src_slot[j] = (int)h->src_dev.size();
         h->src_dev.push_back(d);
     }
@@ -968,12 +968,11 @@ int starmap_set_source(starmap_t* h, int j, const double* q, size_t count) {
     double sq = 0.0;
     for (size_t i = 0; i < np; ++i) sq += q[i] * q[i];
     h->src_sq[j] = sq;
-    if (h->fp32) {
-        std::vector<float> tmp(q, q + np);
-        CK(cudaMemcpy(d, tmp.data(), np * 4, cudaMemcpyHostToDevice), "upload source");
-    } else {
-        CK(cudaMemcpy(d, q, np * 8, cudaMemcpyHostToDevice), "upload source");
-    }
+    std::vector<float> tmp;
+    if (h->fp32) tmp.assign(q, q + np);
+    const size_t row = h->nxg[g] * h->esize;
+    CK(cudaMemcpy2D(d, h->cpg[g] * h->esize, h->fp32 ? (const void*)tmp.data() : (const void*)q, row, row, h->nyg[g],
+                    cudaMemcpyHostToDevice), "upload source");
     // the pass tables only change when a component gains a source
     return new_slot ? rebuild_tables(h) : STARMAP_OK;
 }
@@ -1507,7 +1506,6 @@ void batch_release(starmap_batch_t* b) {
     b->inst.clear();
     if (b->dev_params) cudaFree(b->dev_params);
     if (b->dev_items) cudaFree(b->dev_items);
-    for (GhostJob* g : b->dev_ghosts) if (g) cudaFree(g);
     if (b->dev_off) cudaFree(b->dev_off);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
 }
@@ -1537,9 +1535,8 @@ int batch_sync_params(starmap_batch_t* b) {
 // The pass launches of one starmap_batch_step(b, n) (same schedules as do_steps).
 int batch_issue(starmap_batch_t* b, long n) {
     auto pass = [&](int P, int w) {
-        return tiled_batch_pass(b->dev_params, b->dev_items, b->dev_off, P, w, b->grid, b->smem, b->variant,
-                                b->stream) ||
-               launch_fill_ghosts_jobs(b->dev_ghosts[P], b->nghosts[P], b->stream);
+        return tiled_batch_pass(b->dev_params, b->dev_items, b->dev_off, P, w, b->grid, b->smem, b->shape,
+                                b->stream);
     };
     if (b->schedule == STARMAP_SCHEDULE_MERGED) {
         if (pass(1, 0)) return STARMAP_E_CUDA;
@@ -1704,6 +1701,9 @@ int batch_build(const starmap_config* cfgs, int count, int variant, starmap_batc
     }
     std::vector<BatchShape> shapes;
     b->variant = variant;
+    int max_N = 1;                         // one kernel runs every instance
+    for (int i = 0; i < count; ++i) max_N = std::max(max_N, cfgs[i].N);
+    b->shape = tiled_batch_shape(variant, max_N);
     for (int i = 0; i < count; ++i) {
         starmap_config c = cfgs[i];
         if (c.system != STARMAP_PN2D || c.precision != STARMAP_FP32 || c.closure != STARMAP_CLOSURE_NONE)
@@ -1713,7 +1713,7 @@ int batch_build(const starmap_config* cfgs, int count, int variant, starmap_batc
         c.schedule = b->schedule;
         c.cuda_stream = b->stream;
         starmap_t* h = nullptr;
-        int rc = starmap_create(&c, &h);
+        int rc = create_handle(&c, b->shape, &h);
         if (rc) return bail(bfail(b, rc, "batch instance " + std::to_string(i) + ": " + g_create_error));
         b->inst.push_back(h);
         int tx = 0, ty = 0;
@@ -1727,30 +1727,13 @@ int batch_build(const starmap_config* cfgs, int count, int variant, starmap_batc
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    b->slots = sms * tiled_ctas_per_sm(b->variant);     // resident CTAs of the persistent grid
+    b->slots = sms * tiled_batch_ctas(b->smem, b->shape);   // resident CTAs of the persistent grid
     b->shapes = shapes;
-    int rc = tiled_batch_prepare(b->smem, b->variant);
+    int rc = tiled_batch_prepare(b->smem, b->shape);
     if (rc) return bail(bfail(b, rc, "batch kernel needs more shared memory than the device offers"));
     b->staging.assign((size_t)count * 4 * tiled_params_bytes(), 0);
     b->uploaded.assign(count, ~0ul);
-    // Boundary refresh after a pass of parity P: every component of its two
-    // output grids (even: G11, G22; odd: G21, G12) of every instance.
-    std::vector<GhostJob> jobs[2];
-    for (int P = 0; P < 2; ++P)
-        for (starmap_t* h : b->inst)
-            for (int g : {P ? 1 : 0, P ? 2 : 3})
-                for (int k = 0; k < h->Kg[g]; ++k)
-                    jobs[P].push_back(GhostJob{(float*)h->base[g] + (long)k * h->cstride[g], h->pitch, h->nxg[g],
-                                               h->nyg[g], g, h->p[0], h->p[1], 0});
     e = dev_alloc(&b->dev_params, b->staging.size());
-    for (int P = 0; P < 2 && e == cudaSuccess; ++P) {
-        if (jobs[P].size() > 0x7fffffffu) return bail(bfail(b, STARMAP_E_ARG, "too many components in one batch"));
-        b->nghosts[P] = (int)jobs[P].size();
-        e = dev_alloc(&b->dev_ghosts[P], std::max<size_t>(1, jobs[P].size()) * sizeof(GhostJob));
-        if (e == cudaSuccess && !jobs[P].empty())
-            e = cudaMemcpyAsync(b->dev_ghosts[P], jobs[P].data(), jobs[P].size() * sizeof(GhostJob),
-                                cudaMemcpyHostToDevice, b->stream);
-    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return bail(bfail(b, e == cudaErrorMemoryAllocation ? STARMAP_E_NOMEM : STARMAP_E_CUDA,
                                             std::string("batch setup: ") + cudaGetErrorString(e)));
@@ -1954,8 +1937,8 @@ starmap_t* starmap_batch_instance(starmap_batch_t* b, int i) {
 
 long starmap_batch_launches(const starmap_batch_t* b, long nsteps) {
     if (!b || nsteps <= 0) return 0;
-    // two launches per pass: the batched pass and the boundary refresh
-    return 2 * (b->schedule == STARMAP_SCHEDULE_MERGED ? 2 * nsteps + 1 : 3 * nsteps);
+    // one launch per pass
+    return b->schedule == STARMAP_SCHEDULE_MERGED ? 2 * nsteps + 1 : 3 * nsteps;
 }
 
 int starmap_batch_step(starmap_batch_t* b, long nsteps) {

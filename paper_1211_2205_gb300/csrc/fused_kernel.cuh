@@ -44,9 +44,10 @@ using tiled::f2_fma;
 using tiled::f2_sub;
 using tiled::f2_add;
 using tiled::f2_mul;
+using tiled::add_targets;
+using tiled::load_weights;
 using tiled::lds2;
 using tiled::zero2;
-using tiled::diff_x;
 using tiled::mbar_init;
 using tiled::fence_mbar_init;
 using tiled::mbar_expect_tx;
@@ -57,7 +58,6 @@ using tiled::tma_load_3d;
 using tiled::wait_bounded;
 using tiled::input_shift;
 using tiled::nq_of;
-using tiled::has_imag;
 using tiled::OutGrid;
 
 constexpr int TXO = 62;                 // odd outputs per tile row
@@ -91,13 +91,31 @@ constexpr int PUBLISH = 8;              // E stages between progress publication
 // shortly before) find them in L2
 constexpr int LEAD = 32;
 
+// x-differences of points A (column c) and B (column c + 1) of one box row:
+// right operands at columns c, c + 1, left operands at c - 1, c.  The pair
+// load starts at the even column of the two.
+__device__ __forceinline__ f2 diff_x(const float* row, int c, bool c_even) {
+    if (c_even) {
+        const f2 P = lds2(row + c);                 // v[c], v[c+1]
+        const float Q = row[c - 1];
+        float lo, hi;
+        f2_split(P, lo, hi);
+        return f2_sub(P, f2_make(Q, lo));
+    }
+    const f2 P = lds2(row + c - 1);                 // v[c-1], v[c]
+    const float Q = row[c + 1];
+    float lo, hi;
+    f2_split(P, lo, hi);
+    return f2_sub(f2_make(hi, Q), P);
+}
+
 struct Machine {
     CUtensorMap maps[4];        // input R, input I, old output R, old output I
     OutGrid out[2];             // new values of output kind R, I (the other buffer set)
     int nstages, nin, nfin, nring;
     const int4* stages;
     const float4* coef[2];
-    const int2* fin[2];
+    const int4* fin[2];
     int smem_coef_off[2], smem_fin_off[2], smem_stage_off, smem_part_off, ring_off;
 };
 
@@ -110,7 +128,6 @@ struct FusedParams {
     int tiles_x;
     int N;
     int nclasses;
-    const float* const* srcs;
     int* err;
 };
 
@@ -188,8 +205,11 @@ __device__ __forceinline__ void fused_tiles(const FusedParams& prm, int t0, int 
         for (int k = 0; k < 2; ++k) {
             float4* c = reinterpret_cast<float4*>(smem + m.smem_coef_off[k]);
             for (int i = tid; i < 2 * m.nin; i += THREADS) c[i] = __ldg(m.coef[k] + i);
-            int2* f = reinterpret_cast<int2*>(smem + m.smem_fin_off[k]);
-            for (int i = tid; i < m.nfin; i += THREADS) f[i] = __ldg(m.fin[k] + i);
+            int2* f = reinterpret_cast<int2*>(smem + m.smem_fin_off[k]);     // (offset, has a source)
+            for (int i = tid; i < m.nfin; i += THREADS) {
+                const int4 g = __ldg(m.fin[k] + i);
+                f[i] = make_int2(g.x, (g.z | g.w) != 0);
+            }
         }
         int4* st = reinterpret_cast<int4*>(smem + m.smem_stage_off);
         for (int i = tid; i < m.nstages; i += THREADS) st[i] = __ldg(m.stages + i);
@@ -331,7 +351,7 @@ __device__ __forceinline__ void fused_tiles(const FusedParams& prm, int t0, int 
     input_shift(E ? 0 : 1, 0, px, py, sxR, syR);
     input_shift(E ? 0 : 1, 1, px, py, sxI, syI);
     const OutGrid& G = m.out[K];
-    const long plane = (long)G.nx * G.ny;
+    const long plane = (long)G.cp * G.ny;
     const bool xnode = E ? (K == 1) : (K == 0);          // G22 / G21 have node columns
     const bool ynode = K == 1;                           // G22 / G12 have node rows
     int s = 0, ring_r = 0;
@@ -372,8 +392,8 @@ __device__ __forceinline__ void fused_tiles(const FusedParams& prm, int t0, int 
             };
             plain = stA && stB && gx >= 0 && gx + 1 < G.nx && gy >= 0 && gy < G.ny && !copy(gx) && !copy(gx + 1);
             const int yw = wrap_or_clamp(gy, G.ny, py);
-            cA = (long)yw * G.nx + wrap_or_clamp(gx, G.nx, px);
-            cB = (long)yw * G.nx + wrap_or_clamp(gx + 1, G.nx, px);
+            cA = (long)yw * G.cp + wrap_or_clamp(gx, G.nx, px);
+            cB = (long)yw * G.cp + wrap_or_clamp(gx + 1, G.nx, px);
         }
         const long apos = (long)(gy + 1) * prm.pitch + gx;         // point A inside a component
         f2 ca2[2], cb2[2];
@@ -388,7 +408,8 @@ __device__ __forceinline__ void fused_tiles(const FusedParams& prm, int t0, int 
             cb2[c] = f2_make(b[0], b[1]);
         }
         const float4* cp = reinterpret_cast<const float4*>(smem + m.smem_coef_off[K]);
-        const int2* fp = reinterpret_cast<const int2*>(smem + m.smem_fin_off[K]);
+        const int2* const fp0 = reinterpret_cast<const int2*>(smem + m.smem_fin_off[K]);
+        const int2* fp = fp0;
         auto stage_ptr = [&]() -> const float* {
             if (alive) alive = wait_bounded(&full[ring_r], ring_ph, abort_flag, prm.err);
             return reinterpret_cast<const float*>(ring + ring_r * SB);
@@ -426,11 +447,13 @@ __device__ __forceinline__ void fused_tiles(const FusedParams& prm, int t0, int 
         auto put = [&](float* comp, int x, int y, float v) { comp[(long)(y + 1) * prm.pitch + x] = v; };
         auto finalize = [&](const float* t, f2 W) {
             const int2 f = *fp;
+            const int event = (int)(fp - fp0);
             fp += 1;
             const f2 uo = lds2(t + uoff);
             f2 w = W;
-            if (f.y >= 0) {
-                const float* qs = prm.srcs[f.y];
+            if (f.y != 0) {
+                const int4 g = __ldg(m.fin[K] + event);
+                const float* qs = tiled::source_of(g);
                 w = f2_add(w, f2_make(__ldg(qs + cA), __ldg(qs + cB)));
             }
             const f2 v = f2_fma(aL, uo, f2_mul(bL, w));
@@ -462,26 +485,14 @@ __device__ __forceinline__ void fused_tiles(const FusedParams& prm, int t0, int 
                 }
             }
         };
-        auto accumulate = [&](const float* t, bool inI, f2& Pc, f2& Pn, f2& Nc, f2& Nn) {
-            const float4 cxv = cp[0], cyv = cp[1];
+        // (an absent I input is a box of zeros)
+        auto accumulate = [&](const float* t, f2& Pc, f2& Pn, f2& Nc, f2& Nn) {
+            f2 wx[4], wy[4];
+            load_weights(cp, wx, wy);
             cp += 2;
-            const f2 xPm = f2_make(cxv.x, cxv.x), xP0 = f2_make(cxv.y, cxv.y);
-            const f2 xN0 = f2_make(cxv.z, cxv.z), xNp = f2_make(cxv.w, cxv.w);
-            const f2 yPm = f2_make(cyv.x, cyv.x), yP0 = f2_make(cyv.y, cyv.y);
-            const f2 yN0 = f2_make(cyv.z, cyv.z), yNp = f2_make(cyv.w, cyv.w);
-            f2 dx = diff_x(t + rx, cx, ev);
-            f2 dy = f2_sub(lds2(t + uy), lds2(t + uy - BXI));
-            if (!inI) {
-                if (K == 1) dx = zero2(); else dy = zero2();
-            }
-            Pc = f2_fma(xPm, dx, Pc);
-            Pn = f2_fma(xP0, dx, Pn);
-            Nc = f2_fma(xN0, dx, Nc);
-            Nn = f2_fma(xNp, dx, Nn);
-            Pc = f2_fma(yPm, dy, Pc);
-            Pn = f2_fma(yP0, dy, Pn);
-            Nc = f2_fma(yN0, dy, Nc);
-            Nn = f2_fma(yNp, dy, Nn);
+            const f2 dx = diff_x(t + rx, cx, ev);
+            const f2 dy = f2_sub(lds2(t + uy), lds2(t + uy - BXI));
+            add_targets(dx, dy, wx, wy, Pc, Pn, Nc, Nn);
         };
 
         const int N = prm.N;
@@ -497,9 +508,8 @@ __device__ __forceinline__ void fused_tiles(const FusedParams& prm, int t0, int 
             f2 Pc = zero2(), Nc = zero2(), Pn, Nn;
             auto qstep = [&](int q, f2& Pc_, f2& Nc_, f2& Pn_, f2& Nn_) {
                 Pn_ = q < nqload ? pp[q * ncons] : zero2();
-                Nn_ = zero2();
                 const float* t = stage_ptr();
-                accumulate(t, has_imag(lp, q), Pc_, Pn_, Nc_, Nn_);
+                accumulate(t, Pc_, Pn_, Nc_, Nn_);
                 if (q >= 1 && q - 1 < nqp) finalize(t, Pc_);
                 stage_done();
                 if (q < nqn) pp[q * ncons] = Nc_;

@@ -50,7 +50,8 @@ struct GridDev {
     T* base = nullptr;            // point (0, 0) of component 0
     long cstride = 0;             // elements between components
     int nx = 0, ny = 0, K = 0;    // points and components of this grid
-    T* coef = nullptr;            // decay coefficients [cls][4][ny][nx]
+    T* coef = nullptr;            // decay coefficients [cls][4][ny][cp]
+    int cp = 0;                   // row pitch of the coefficients and sources (a multiple of 32, >= nx)
 };
 
 // One output component of the gather pass.
@@ -72,7 +73,7 @@ struct GatherArgs {
     int which;                    // 0: half-step coefficients, 1: full step
     const GatherOut* outs;
     const GatherCoef<T>* coefs;
-    T* const* src;                // source arrays [ny][nx] by slot
+    T* const* src;                // source arrays [ny][cp] by slot
 };
 
 template <class T>
@@ -93,17 +94,6 @@ struct GhostPassArgs {
     int p[2];
 };
 
-// Boundary copies of one FP32 component, one entry of a batched refresh
-// (comp points at the component's first interior value, as GridDev::base).
-struct GhostJob {
-    float* comp;
-    long pitch;
-    int nx, ny;
-    int grid;                     // grid number (its x / y type)
-    int px, py;                   // periodic in x / y
-    int pad;
-};
-
 template <class T>
 struct ReduceArgs {
     GridDev<T> g[4];
@@ -117,7 +107,6 @@ template <class T> int launch_gather_pass(const GatherArgs<T>& a, void* stream);
 template <class T> int launch_fill_ghosts(const GhostArgs<T>& a, void* stream);
 // overlap: programmatic dependent launch (after a short tiled pass)
 template <class T> int launch_fill_ghosts_pass(const GhostPassArgs<T>& a, void* stream, bool overlap);
-int launch_fill_ghosts_jobs(const GhostJob* jobs, int njobs, void* stream);
 template <class T> int launch_reduce(const ReduceArgs<T>& a, double* partials, int nblocks,
                                      double* result, void* stream);
 template <class T> int launch_axpby(T* out, const T* x, const T* y, double alpha, double beta,

@@ -145,8 +145,8 @@ __global__ void k_gather_pass(const GatherArgs<T> A) {
     const long o_r = (long)(iy + 1) * pitch + xr;
     const long o_u = (long)(yu + 1) * pitch + ix;
     const long o_self = (long)(iy + 1) * pitch + ix;
-    const long cidx = (long)iy * G.nx + ix;
-    const long plane = (long)G.nx * G.ny;
+    const long cidx = (long)iy * G.cp + ix;
+    const long plane = (long)G.cp * G.ny;
     const T* Xb = A.g[xg].base;
     const T* Yb = A.g[yg].base;
     const long cxs = A.g[xg].cstride, cys = A.g[yg].cstride;
@@ -215,17 +215,6 @@ __global__ void k_fill_ghosts_pass(const GhostPassArgs<T> A) {
     const int items = ghost_items<T>(nx, ny, A.p[0] || !xnode, A.p[1] || !ynode);
     for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < items; r += gridDim.x * blockDim.x)
         ghost_item(comp, A.pitch, nx, ny, xnode, ynode, A.p[0], A.p[1], r);
-}
-
-// Batched refresh: block b re-stores the boundary points of component
-// jobs[b] with their copies.
-__global__ void k_fill_ghosts_jobs(const GhostJob* __restrict__ jobs) {
-    const GhostJob J = jobs[blockIdx.x];
-    const bool xnode = (J.grid & 1) != 0, ynode = (J.grid & 2) != 0;
-    const int nx = J.nx, ny = J.ny;
-    const int items = ghost_items<float>(nx, ny, J.px || !xnode, J.py || !ynode);
-    for (int r = threadIdx.x; r < items; r += blockDim.x)
-        ghost_item(J.comp, J.pitch, nx, ny, xnode, ynode, J.px, J.py, r);
 }
 
 // Deterministic FP64 reduction: per-block partials (mass, sum of squares,
@@ -339,12 +328,6 @@ int launch_fill_ghosts_pass(const GhostPassArgs<T>& a, void* stream, bool overla
     const dim3 grid((len + 255) / 256, K);
     const cudaError_t e = launch_pdl(k_fill_ghosts_pass<T>, grid, dim3(256), 0, (cudaStream_t)stream, overlap, a);
     return status_of(e != cudaSuccess ? e : cudaGetLastError());
-}
-
-int launch_fill_ghosts_jobs(const GhostJob* jobs, int njobs, void* stream) {
-    if (njobs <= 0) return 0;
-    k_fill_ghosts_jobs<<<njobs, 256, 0, (cudaStream_t)stream>>>(jobs);
-    return status_of(cudaGetLastError());
 }
 
 template <class T>

@@ -11,27 +11,13 @@
 
 #include "internal.h"
 #include "tiled.h"
-// the kernels, once per tile height (namespaces tiled: 10 rows, two per
-// consumer warp; tiled5: 5 rows, one per consumer warp)
-#include "tiled_kernel.cuh"
-#undef STARMAP_TILED_NS
-#undef STARMAP_TILED_TY
-#undef STARMAP_TILED_MINB
-#undef STARMAP_TILED_RW
-#define STARMAP_TILED_NS tiled5
-#define STARMAP_TILED_TY 5
-#define STARMAP_TILED_MINB 2
-#define STARMAP_TILED_RW 1
 #include "tiled_kernel.cuh"
 // the temporally fused step (even then odd update per tile, one launch)
 #include "fused_kernel.cuh"
 
 namespace starmap {
 
-using namespace tiled;   // constants and types common to both tile heights
-
-static_assert(sizeof(tiled::Params) == sizeof(tiled5::Params), "both tile heights share the parameter layout");
-static_assert(tiled::TX == tiled5::TX && tiled::BX == tiled5::BX, "both tile heights share the tile width");
+using namespace tiled;
 
 namespace {
 
@@ -85,27 +71,64 @@ struct PassTables {
     std::vector<float> coef;              // nin x 16 (each coefficient twice, for f32x2)
     std::vector<int2> fin;                // (local, class)
     std::vector<int> fin_comp;            // global component per finalise event
+    std::vector<char> heads;              // per stage: the first of an input order (nothing to finalise)
     int nin = 0;
     int top = 0;                          // highest output order finalised
 };
 
-// Orders up to this use the 5-row tiles by default (few stages per tile:
-// two CTAs per SM hide each other's setup, fill and drain).
-constexpr int SHORT_TILE_MAX_N = 3;
+// Highest order of the 10-row tiles: beyond it their tables leave no room
+// for a ring.
+constexpr int TALL_TILE_MAX_N = 55;
+// Highest order whose 10-row tiles keep each weight twice in shared memory.
+constexpr int TALL_DUP_MAX_N = 49;
+// Highest order of the five-row bands (below): two of their CTAs fit an SM.
+constexpr int WIDE_BAND_MAX_N = 15;
 
-// Per tile height: rows, input box rows, threads, consumer threads, point
-// pairs per consumer thread, bytes of a ring stage.
-struct Variant { int ty, byi, threads, consumers, pp, stage_bytes; };
-const Variant kVariant[2] = {
-    {tiled::TY, tiled::BYI, tiled::THREADS, tiled::CONSUMERS, tiled::PP, tiled::STAGE_BYTES},
-    {tiled5::TY, tiled5::BYI, tiled5::THREADS, tiled5::CONSUMERS, tiled5::PP, tiled5::STAGE_BYTES}};
-static_assert(tiled::MAX_STAGES == tiled5::MAX_STAGES && tiled::RING_OFF == tiled5::RING_OFF,
-              "both tile heights share the barrier area");
-// Ring depth: as many stages as the shared memory allows, at most RING_DEPTH
-// (measured with 6, 9, 12 and 15 stages: 9 is best or level at every order
-// and grid tried; 15 costs 5 % at N = 13..15), at least MIN_RING.
+// Per tile shape: rows, input box rows, threads, bytes of the partial sums
+// of one q, of a ring stage and of a stage record, resident CTAs per SM, the
+// kernels.
+struct Variant {
+    int ty, byi, threads, part_bytes, stage_bytes, rec_bytes, minb;
+    void (*pass)(Params, int);
+    void (*batch)(const Params*, const int4*, const int*, int, int);
+};
+// 10-row tiles as two bands of five rows, two CTAs per SM: the fewest
+// instructions per point, for grids with more tiles than SMs at orders up to
+// WIDE_BAND_MAX_N; as five bands of two rows, one CTA per SM: more warps on a
+// tile, for the higher orders, whose partial sums leave room for one CTA, and
+// for grids of at most a tile per SM, where the latency of a tile's chain of
+// stages is the pass (and, lean, with each weight kept once).  Measured, us
+// per pass, two-row / five-row bands: N = 3 at 1024^2 24.8 / 18.7, N = 13 at
+// 512^2 47.9 / 39.2, N = 9 at 1501 x 1099 109 / 103, N = 15 at 350^2 31.7 /
+// 26.1, but N = 5 at 256^2 5.2 / 6.5, N = 21 at 300^2 50 / 65, N = 39 at
+// 1024^2 865 / 940.
+// 5-row tiles: one row per warp, two CTAs per SM.
+enum { TALL_WIDE, TALL, TALL_LEAN, SHORT, SHAPES };
+template <class S>
+Variant variant_of() {
+    return {S::TY, S::BYI, S::THREADS, S::PART_BYTES, S::STAGE_BYTES, S::REC_BYTES, S::MINB, k_tiled_pass<S>, k_tiled_batch<S>};
+}
+const Variant kVariant[SHAPES] = {variant_of<Shape<5, 2, 2, true>>(), variant_of<Shape<2, 5, 1, true>>(),
+                                  variant_of<Shape<2, 5, 1, false>>(), variant_of<Shape<1, 5, 2, true>>()};
+
+int shape_of(int variant, int N, long tiles, int sms) {
+    if (variant) return SHORT;
+    if (N <= WIDE_BAND_MAX_N && tiles > sms) return TALL_WIDE;
+    return N <= TALL_DUP_MAX_N ? TALL : TALL_LEAN;
+}
+
+int sm_count() {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 1;
+    return sms;
+}
+
+// Ring depth: as many stages as the shared memory allows, at most RING_DEPTH,
+// at least MIN_RING (GOOD_RING before another CTA per SM is given room).
 constexpr int RING_DEPTH = 9;
-constexpr int MIN_RING = 4;
+constexpr int GOOD_RING = 4;
+constexpr int MIN_RING = 3;
 static_assert(RING_DEPTH <= MAX_STAGES, "the barrier area holds the ring");
 
 }  // namespace
@@ -120,11 +143,14 @@ struct TiledPlan {
     CUtensorMap maps_in[4], maps_out[4];
     PassTables tab[2];
     void* dev_stages[2] = {nullptr, nullptr};
+    void* dev_rec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};    // [P][K]
+    // the fused step's tables
+    int nin[2] = {0, 0}, nfin[2] = {0, 0};
     void* dev_coef[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};   // [P][K]
     void* dev_fin[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
-    void* dev_src = nullptr;
     int tiles_x = 0, tiles_y = 0;
     int variant = 0;                      // 0: 10-row tiles, 1: 5-row tiles
+    int shape = 0;                        // index into kVariant
     int sms = 1;
     int ctas_per_sm = 1;                  // resident CTAs per SM the tables allow (<= the variant's)
     int smem_bytes[2] = {0, 0};
@@ -150,11 +176,10 @@ void free_tables(TiledPlan* pl) {
         for (int K = 0; K < 2; ++K) {
             if (pl->dev_coef[P][K]) cudaFree(pl->dev_coef[P][K]);
             if (pl->dev_fin[P][K]) cudaFree(pl->dev_fin[P][K]);
-            pl->dev_coef[P][K] = pl->dev_fin[P][K] = nullptr;
+            if (pl->dev_rec[P][K]) cudaFree(pl->dev_rec[P][K]);
+            pl->dev_coef[P][K] = pl->dev_fin[P][K] = pl->dev_rec[P][K] = nullptr;
         }
     }
-    if (pl->dev_src) cudaFree(pl->dev_src);
-    pl->dev_src = nullptr;
     if (pl->dev_odep) cudaFree(pl->dev_odep);
     pl->dev_odep = nullptr;
     pl->fready = false;
@@ -253,10 +278,12 @@ bool build_pass(TiledPlan* pl, const SystemMatrices& sys, const std::vector<int>
             ok = ok && emit_input_pair(lp, q);
             if (q >= 1 && q - 1 < nqp) ok = ok && emit_fin_pair(lp - 1, q - 1);
             close_stage();
+            t.heads.push_back(q == 0);
         }
         if (ok && nq - 1 < nqp) {
             ok = ok && emit_fin_pair(lp - 1, nq - 1);
             close_stage();
+            t.heads.push_back(0);
         }
     }
     const int L = last_in + 1;
@@ -264,6 +291,7 @@ bool build_pass(TiledPlan* pl, const SystemMatrices& sys, const std::vector<int>
         for (int q = 0; q < nq_of(L) && ok; ++q) {
             ok = ok && emit_fin_pair(L, q);
             close_stage();
+            t.heads.push_back(0);
         }
     if (!ok) { err = "moment placement differs from the tiled kernel's"; return false; }
     // every component of the output parity is finalised exactly once
@@ -323,9 +351,9 @@ int build_fused(TiledPlan* pl) {
         const Params& q = pl->prm[M == 0 ? 0 : 1][1];
         for (int K = 0; K < 2; ++K) {
             coef_rel[M][K] = tab;
-            tab = al16(tab + q.nin * 2 * (int)sizeof(float4));
+            tab = al16(tab + pl->nin[M] * 2 * (int)sizeof(float4));
             fin_rel[M][K] = tab;
-            tab = al16(tab + q.nfin * (int)sizeof(int2));
+            tab = al16(tab + pl->nfin[M] * (int)sizeof(int2));   // staged as (offset, has a source)
         }
         stage_rel[M] = tab;
         tab = al16(tab + q.nstages * (int)sizeof(int4));
@@ -385,14 +413,15 @@ int build_fused(TiledPlan* pl) {
                 m.out[k].coef = (const float*)pl->coef[g];
                 m.out[k].nx = pl->geo.nx[g];
                 m.out[k].ny = pl->geo.ny[g];
-                m.coef[k] = q.coef[k];
-                m.fin[k] = q.fin[k];
+                m.out[k].cp = pl->geo.cp[g];
+                m.coef[k] = (const float4*)pl->dev_coef[P][k];
+                m.fin[k] = (const int4*)pl->dev_fin[P][k];
                 m.smem_coef_off[k] = tables + coef_rel[M][k];
                 m.smem_fin_off[k] = tables + fin_rel[M][k];
             }
             m.nstages = q.nstages;
-            m.nin = q.nin;
-            m.nfin = q.nfin;
+            m.nin = pl->nin[P];
+            m.nfin = pl->nfin[P];
             m.nring = depth;
             m.stages = q.stages;
             m.smem_stage_off = tables + stage_rel[M];
@@ -407,7 +436,6 @@ int build_fused(TiledPlan* pl) {
         fp.tiles_x = pl->ftiles_x;
         fp.N = pl->N;
         fp.nclasses = pl->nclasses;
-        fp.srcs = (const float* const*)pl->dev_src;
         fp.err = pl->err_dev;
     }
     pl->fready = true;
@@ -454,22 +482,19 @@ int tiled_create(const TiledGeometry& geo, TiledPlan** out) {
     *out = pl;
     if (geo.N < 1 || geo.N > MAXN) { pl->err = "tiled kernel supports 1 <= N <= 63"; return -8; }
     pl->variant = geo.variant == 1 ? 1 : 0;
-    const Variant& V = kVariant[pl->variant];
+    int nxmax = 0, nymax = 0;
+    for (int g = 0; g < 4; ++g) { nxmax = std::max(nxmax, geo.nx[g]); nymax = std::max(nymax, geo.ny[g]); }
+    pl->sms = sm_count();
+    pl->tiles_x = (nxmax + TX - 1) / TX;
+    pl->shape = geo.shape >= 0 ? geo.shape : shape_of(pl->variant, geo.N, (long)pl->tiles_x * ((nymax + 9) / 10), pl->sms);
+    const Variant& V = kVariant[pl->shape];
+    pl->tiles_y = (nymax + V.ty - 1) / V.ty;
     for (int g = 0; g < 4; ++g) {
         if (!encode_grid_map(&pl->maps_in[g], geo.base[g], geo.pitch, geo.rows, geo.K[g], BX, V.byi) ||
             !encode_grid_map(&pl->maps_out[g], geo.base[g], geo.pitch, geo.rows, geo.K[g], TX, V.ty)) {
             pl->err = "cuTensorMapEncodeTiled failed";
             return -4;
         }
-    }
-    int nxmax = 0, nymax = 0;
-    for (int g = 0; g < 4; ++g) { nxmax = std::max(nxmax, geo.nx[g]); nymax = std::max(nymax, geo.ny[g]); }
-    pl->tiles_x = (nxmax + TX - 1) / TX;
-    pl->tiles_y = (nymax + V.ty - 1) / V.ty;
-    {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&pl->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || pl->sms < 1) pl->sms = 1;
     }
     if (dev_alloc(&pl->err_dev, sizeof(int)) != cudaSuccess || cudaMemset(pl->err_dev, 0, sizeof(int)) != cudaSuccess) {
         pl->err = "cudaMalloc error flag failed";
@@ -483,10 +508,9 @@ int tiled_update(TiledPlan* pl, const SystemMatrices& sys, const std::vector<int
                  const std::vector<char>& frozen, double dx, double dy) {
     free_tables(pl);
     pl->ready = false;
-    {
-        std::vector<const float*> sp(src_dev.size());
-        for (size_t i = 0; i < src_dev.size(); ++i) sp[i] = (const float*)src_dev[i];
-        if (!upload(&pl->dev_src, sp)) { pl->err = "uploading the source table failed"; return -4; }
+    if (pl->variant == 0 && pl->N > TALL_TILE_MAX_N) {
+        pl->err = "tiled kernel needs more shared memory than the device offers";
+        return -8;
     }
     const int gin[2][2] = {{1, 2}, {0, 3}};
     const int gout[2][2] = {{0, 3}, {1, 2}};
@@ -494,7 +518,7 @@ int tiled_update(TiledPlan* pl, const SystemMatrices& sys, const std::vector<int
         PassTables& t = pl->tab[P];
         if (!build_pass(pl, sys, comp_class, frozen, P, dx, dy, t, pl->err)) return -8;
         // per output kind K: coefficient rows (x part of the kind-K input,
-        // y part of the other input) and finalise entries (offset, source slot)
+        // y part of the other input) and finalise entries (offset, source address)
         // (each value once: the kernel pairs it for f32x2 itself)
         const size_t nsteps = t.coef.size() / 32;
         std::vector<float> ck[2];
@@ -509,11 +533,11 @@ int tiled_update(TiledPlan* pl, const SystemMatrices& sys, const std::vector<int
                 }
             }
         }
-        std::vector<int2> fk[2];
+        std::vector<int4> fk[2];
         for (size_t e = 0; e + 1 < t.fin.size() + 1; e += 2) {
             for (int K = 0; K < 2; ++K) {
                 const int comp = t.fin_comp[e + K];
-                if (comp < 0 || frozen[comp]) { fk[K].push_back(make_int2(-1, -1)); continue; }
+                if (comp < 0 || frozen[comp]) { fk[K].push_back(make_int4(-1, 0, 0, 0)); continue; }
                 // the component's element offset in units of 32 (pitch, and so the
                 // component stride, is a multiple of 32): 2^36 values per grid
                 const int g = gout[P][K];
@@ -522,7 +546,8 @@ int tiled_update(TiledPlan* pl, const SystemMatrices& sys, const std::vector<int
                     pl->err = "state too large for the tiled kernel's offsets";
                     return -8;
                 }
-                fk[K].push_back(make_int2((int)(off / 32), src_slot[comp]));
+                const unsigned long long src = src_slot[comp] >= 0 ? (unsigned long long)(uintptr_t)src_dev[src_slot[comp]] : 0;
+                fk[K].push_back(make_int4((int)(off / 32), 0, (int)(unsigned)src, (int)(unsigned)(src >> 32)));
             }
         }
         for (int K = 0; K < 2; ++K)
@@ -530,59 +555,77 @@ int tiled_update(TiledPlan* pl, const SystemMatrices& sys, const std::vector<int
                 pl->err = "uploading the tiled tables failed";
                 return -4;
             }
-        if (!upload(&pl->dev_stages[P], t.stages)) {
+        pl->nin[P] = (int)nsteps;
+        pl->nfin[P] = (int)fk[0].size();
+        // an absent I input is loaded as a box of zeros: a component outside the tensor
+        std::vector<int4> st = t.stages;
+        for (int4& v : st)
+            if (v.x >= 0 && v.y < 0) v.y = std::max(1, pl->geo.K[gin[P][1]]);
+        if (!upload(&pl->dev_stages[P], st)) {
             pl->err = "uploading the tiled tables failed";
             return -4;
         }
-        // shared memory: barriers, ring, coefficient rows, finalise events,
-        // partial sums; the ring takes what the variant's CTAs per SM leave,
-        // up to RING_DEPTH stages (a deeper ring keeps more loads in flight:
-        // 9 stages instead of 6 made the P_39 1024^2 pass 7 % faster)
-        const Variant& V = kVariant[pl->variant];
-        int tables = 0;
-        int coef_rel[2], fin_rel[2];
+        // per output kind, a record per stage (Params::rec)
+        std::vector<float> rk[2];
         for (int K = 0; K < 2; ++K) {
-            coef_rel[K] = tables;
-            tables += (int)(ck[K].size() * sizeof(float));
-            tables = (tables + 15) & ~15;
-            fin_rel[K] = tables;
-            tables += (int)(fk[K].size() * sizeof(int2));
-            tables = (tables + 15) & ~15;
+            size_t in = 0, fin = 0;                 // inputs and finalise entries so far
+            bool prev = false;                      // the stage before had an input of the same order
+            for (size_t k = 0; k < t.stages.size(); ++k) {
+                const bool has_in = t.stages[k].x >= 0;
+                const float* p = prev ? ck[K].data() + 8 * (in - 1) : nullptr;
+                const float* c = has_in ? ck[K].data() + 8 * in : nullptr;
+                float row[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                if (p && !t.heads[k]) { row[0] = p[1]; row[1] = p[5]; row[2] = p[3]; row[3] = p[7]; }
+                if (c) { row[4] = c[0]; row[5] = c[4]; row[6] = c[2]; row[7] = c[6]; }
+                int4 f = make_int4(-1, 0, 0, 0);
+                if (!t.heads[k]) f = fk[K][fin++];
+                if (has_in && !t.heads[k] && f.x < 0) {
+                    pl->err = "the tiled kernel needs every target below the top order";
+                    return -8;
+                }
+                rk[K].insert(rk[K].end(), row, row + 8);
+                const int fi[4] = {f.x, f.y, f.z, f.w};
+                float ff[4];
+                std::memcpy(ff, fi, sizeof(ff));
+                rk[K].insert(rk[K].end(), ff, ff + 4);
+                prev = has_in;
+                in += has_in;
+            }
+            if (in != nsteps || fin != fk[K].size()) { pl->err = "tiled stage list and tables differ"; return -8; }
+            if (!upload(&pl->dev_rec[P][K], rk[K])) { pl->err = "uploading the tiled tables failed"; return -4; }
         }
-        const int stage_rel = tables;
+        // shared memory: barriers, partial sums, records, stages, ring.  The
+        // ring takes what the resident CTAs leave
+        const Variant& V = kVariant[pl->shape];
+        int tables = PART_OFF + nq_of(pl->N) * V.part_bytes;
+        int rec_off[2];
+        for (int K = 0; K < 2; ++K) {
+            rec_off[K] = tables;
+            tables += (int)t.stages.size() * V.rec_bytes;
+        }
+        const int stage_off = tables;
         tables += (int)(t.stages.size() * sizeof(int4));
-        tables = (tables + 15) & ~15;
-        const int part_rel = tables;
-        tables += nq_of(pl->N) * V.pp * V.consumers * 8;    // pp pairs of partial sums per consumer thread and q
+        const int ring_off = (tables + 127) & ~127;
         int dev = 0, maxsm = 0, persm = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
         cudaDeviceGetAttribute(&persm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-        // per-CTA budget: the variant's CTAs per SM (1 KB reserved per CTA),
-        // less the batch kernel's static parameter copy; where the tables of
-        // a high order do not leave room for the ring, one CTA per SM
-        auto ring_for = [&](int minb) {
-            const int budget = std::min(maxsm, persm / minb - 1024) - (int)sizeof(Params) - 256;
-            return std::min(RING_DEPTH, (budget - RING_OFF - tables) / V.stage_bytes);
+        // per-CTA budget at c CTAs per SM (1 KB reserved per CTA), less the
+        // batch kernel's static parameter copy
+        auto ring_for = [&](int c) {
+            const int budget = std::min(maxsm, persm / c - 1024) - (int)sizeof(Params) - 256;
+            return std::min(RING_DEPTH, (budget - ring_off) / V.stage_bytes);
         };
-        int minb = tiled_ctas_per_sm(pl->variant);
-        int nring = ring_for(minb);
-        if (nring < MIN_RING && minb > 1) {
-            minb = 1;
-            nring = ring_for(1);
-        }
+        int minb = V.minb;
+        if (P == 1) minb = pl->ctas_per_sm;         // (both parities at the same residency)
+        while (minb > 1 && ring_for(minb) < GOOD_RING) --minb;
+        const int nring = ring_for(minb);
         if (nring < MIN_RING) { pl->err = "tiled kernel needs more shared memory than the device offers"; return -8; }
-        pl->ctas_per_sm = P == 0 ? minb : std::min(pl->ctas_per_sm, minb);
-        const int ring_end = RING_OFF + nring * V.stage_bytes;
-        const int coef_off[2] = {ring_end + coef_rel[0], ring_end + coef_rel[1]};
-        const int fin_off[2] = {ring_end + fin_rel[0], ring_end + fin_rel[1]};
-        const int stage_off = ring_end + stage_rel, part_off = ring_end + part_rel;
-        pl->smem_bytes[P] = ring_end + tables;
+        pl->ctas_per_sm = minb;
+        pl->smem_bytes[P] = ring_off + nring * V.stage_bytes;
         pl->nring[P] = nring;
-        const int need = std::max(pl->smem_bytes[0], pl->smem_bytes[1]);
-        const cudaError_t fe = pl->variant
-            ? cudaFuncSetAttribute(tiled5::k_tiled_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, need)
-            : cudaFuncSetAttribute(tiled::k_tiled_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, need);
+        // (the function's limit, common to every handle: not this plan's need)
+        const cudaError_t fe = cudaFuncSetAttribute(V.pass, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm);
         if (fe != cudaSuccess) {
             pl->err = "cudaFuncSetAttribute failed";
             return -4;
@@ -599,40 +642,39 @@ int tiled_update(TiledPlan* pl, const SystemMatrices& sys, const std::vector<int
                 prm.out[k].coef = (const float*)pl->coef[g];
                 prm.out[k].nx = pl->geo.nx[g];
                 prm.out[k].ny = pl->geo.ny[g];
+                prm.out[k].cp = pl->geo.cp[g];
             }
             prm.pitch = pl->geo.pitch;
             prm.p[0] = pl->geo.p[0];
             prm.p[1] = pl->geo.p[1];
             prm.tiles_x = pl->tiles_x;
+            prm.skew = 1;
             prm.N = pl->N;
             prm.P = P;
             prm.which = w;
             prm.nclasses = pl->nclasses;
             prm.nstages = (int)t.stages.size();
-            prm.nin = (int)nsteps;
-            prm.nfin = (int)fk[0].size();
             prm.nring = nring;
             prm.top = t.top;
             prm.stages = (const int4*)pl->dev_stages[P];
             for (int K = 0; K < 2; ++K) {
-                prm.coef[K] = (const float4*)pl->dev_coef[P][K];
-                prm.fin[K] = (const int2*)pl->dev_fin[P][K];
-                prm.smem_coef_off[K] = coef_off[K];
-                prm.smem_fin_off[K] = fin_off[K];
+                prm.rec[K] = (const float4*)pl->dev_rec[P][K];
+                prm.smem_rec_off[K] = rec_off[K];
             }
-            prm.srcs = (const float* const*)pl->dev_src;
             prm.err = pl->err_dev;
-            prm.smem_part_off = part_off;
             prm.smem_stage_off = stage_off;
+            prm.smem_ring_off = ring_off;
             for (int K = 0; K < 2; ++K) {
-                int slot = -1;
+                unsigned long long src = 0;
                 bool one = true;
-                for (const int2& f : fk[K])
-                    if (f.y >= 0) {
-                        if (slot >= 0 && f.y != slot) one = false;
-                        slot = f.y;
+                for (const int4& f : fk[K])
+                    if ((f.z | f.w) != 0) {
+                        const unsigned long long a = ((unsigned long long)(unsigned)f.w << 32) | (unsigned)f.z;
+                        if (src != 0 && a != src) one = false;
+                        src = a;
                     }
-                prm.pf_src[K] = slot >= 0 && one ? (const float*)src_dev[slot] : nullptr;
+                prm.any_src[K] = src != 0;
+                prm.pf_src[K] = one ? (const float*)(uintptr_t)src : nullptr;
             }
         }
     }
@@ -719,15 +761,9 @@ int tiled_pass(TiledPlan* pl, bool odd, int which, void* stream) {
     // tables while the previous kernel of the stream finishes
     const bool pdl = tiled_overlap(pl, odd);
     cudaError_t e;
-    if (pl->variant) {
-        tiled5::Params q;
-        std::memcpy(&q, &pl->prm[P][which], sizeof(q));
-        e = launch_pdl(tiled5::k_tiled_pass, dim3(grid), dim3(tiled5::THREADS), (size_t)pl->smem_bytes[P],
-                       (cudaStream_t)stream, pdl, q, ntiles);
-    } else {
-        e = launch_pdl(tiled::k_tiled_pass, dim3(grid), dim3(tiled::THREADS), (size_t)pl->smem_bytes[P],
-                       (cudaStream_t)stream, pdl, pl->prm[P][which], ntiles);
-    }
+    const Variant& V = kVariant[pl->shape];
+    e = launch_pdl(V.pass, dim3(grid), dim3(V.threads), (size_t)pl->smem_bytes[P],
+                   (cudaStream_t)stream, pdl, pl->prm[P][which], ntiles);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {
         pl->err = std::string("tiled pass launch: ") + cudaGetErrorString(e);
@@ -759,7 +795,10 @@ int tiled_export_params(TiledPlan* pl, void* host4) {
     if (!pl || !pl->ready) return -7;
     Params* d = static_cast<Params*>(host4);
     for (int P = 0; P < 2; ++P)
-        for (int w = 0; w < 2; ++w) d[2 * P + w] = pl->prm[P][w];
+        for (int w = 0; w < 2; ++w) {
+            d[2 * P + w] = pl->prm[P][w];
+            d[2 * P + w].skew = 0;          // strips of a batch stay in their column
+        }
     return 0;
 }
 
@@ -806,30 +845,39 @@ int tiled_wait_selftest(int* gave_up) {
     return 0;
 }
 
-int tiled_default_variant(int N) { return N <= SHORT_TILE_MAX_N ? 1 : 0; }
+int tiled_default_variant(int N, int nx, int ny) {
+    // 5-row tiles where the 10-row ones would leave half the SMs without a
+    // tile: P_39 on 150^2 (45 tiles) 164 us per pass instead of 180
+    const long tiles = (long)((nx + TX - 1) / TX) * ((ny + 9) / 10);
+    return N > TALL_TILE_MAX_N || 2 * tiles <= sm_count() ? 1 : 0;
+}
 
-int tiled_ctas_per_sm(int variant) { return variant ? tiled5::MINB : tiled::MINB; }
+int tiled_batch_shape(int variant, int max_N) { return shape_of(variant, max_N, 1 << 30, 1); }
 
-int tiled_batch_prepare(int smem_bytes, int variant) {
+int tiled_batch_ctas(int smem_bytes, int shape) {
+    int dev = 0, persm = 0;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&persm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess) return 1;
+    // 1 KB reserved per CTA, and the kernel's static parameter copy
+    const int fit = persm / (smem_bytes + (int)sizeof(Params) + 256 + 1024);
+    return std::max(1, std::min(kVariant[shape].minb, fit));
+}
+
+int tiled_batch_prepare(int smem_bytes, int shape) {
     int dev = 0, maxsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (smem_bytes + (int)sizeof(Params) > maxsm) return -8;
-    const cudaError_t e = variant
-        ? cudaFuncSetAttribute(tiled5::k_tiled_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes)
-        : cudaFuncSetAttribute(tiled::k_tiled_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+    const cudaError_t e = cudaFuncSetAttribute(kVariant[shape].batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               maxsm - (int)sizeof(Params));
     return e == cudaSuccess ? 0 : -4;
 }
 
 int tiled_batch_pass(const void* params, const void* items, const int* off, int P, int which, int grid,
-                     int smem_bytes, int variant, void* stream) {
+                     int smem_bytes, int shape, void* stream) {
     if (grid <= 0) return 0;
-    if (variant)
-        tiled5::k_tiled_batch<<<grid, tiled5::THREADS, smem_bytes, (cudaStream_t)stream>>>(
-            static_cast<const tiled5::Params*>(params), static_cast<const int4*>(items), off, P, which);
-    else
-        tiled::k_tiled_batch<<<grid, tiled::THREADS, smem_bytes, (cudaStream_t)stream>>>(
-            static_cast<const tiled::Params*>(params), static_cast<const int4*>(items), off, P, which);
+    kVariant[shape].batch<<<grid, kVariant[shape].threads, smem_bytes, (cudaStream_t)stream>>>(
+        static_cast<const Params*>(params), static_cast<const int4*>(items), off, P, which);
     return cudaGetLastError() == cudaSuccess ? 0 : -4;
 }
 

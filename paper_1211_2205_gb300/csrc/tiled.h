@@ -13,14 +13,18 @@ struct TiledGeometry {
     void* base[4];
     long cstride[4];
     int nx[4], ny[4], K[4];
+    int cp[4];                         // row pitch of the decay coefficients and sources
     long pitch, rows;
     int p[2];
     int N;
-    int variant = 0;                   // tile height: 0 = 10 rows (one CTA per SM), 1 = 5 rows (two per SM)
+    int variant = 0;                   // tile height: 0 = 10 rows, 1 = 5 rows
+    int shape = -1;                    // tile shape, or -1 for the one the height, order and grid ask for
+                                       // (the instances of a batch share one: tiled_batch_shape)
 };
 
-// Tile height the tiled kernel uses for order N when nothing else decides.
-int tiled_default_variant(int N);
+// Tile height the tiled kernel uses for order N on nx x ny points when
+// nothing else decides.
+int tiled_default_variant(int N, int nx, int ny);
 
 bool tiled_supported(int system, int N, int precision);
 // Host only: the stage list of pass P (parity of its outputs) as global
@@ -36,9 +40,8 @@ int tiled_update(TiledPlan* plan, const SystemMatrices& sys, const std::vector<i
                  const std::vector<char>& frozen, double dx, double dy);
 void tiled_set_coef(TiledPlan* plan, int g, void* coef, int nclasses);
 int tiled_pass(TiledPlan* plan, bool odd, int which, void* stream);
-// Whether the pass is launched with programmatic dependent launch (so its
-// boundary refresh should be too): only for short passes, where the kernel
-// boundary is a visible share of the pass.
+// Whether the pass is launched with programmatic dependent launch: only for
+// short passes, where the kernel boundary is a visible share of the pass.
 bool tiled_overlap(TiledPlan* plan, bool odd);
 // Temporally fused step: one launch applies the full even update and then
 // the full odd update, tile by tile (fused_kernel.cuh), reading one buffer
@@ -56,8 +59,7 @@ void tiled_destroy(TiledPlan* plan);
 
 // Batched passes over several plans (one persistent launch per pass).
 size_t tiled_params_bytes();
-// Copy the plan's four pass parameter blocks (index 2 P + which) to host4
-// (the passes leave the boundary copies to a separate refresh).
+// Copy the plan's four pass parameter blocks (index 2 P + which) to host4.
 int tiled_export_params(TiledPlan* plan, void* host4);
 int tiled_smem_bytes(TiledPlan* plan, int P);
 void tiled_tile_grid(TiledPlan* plan, int* tiles_x, int* tiles_y);
@@ -66,16 +68,18 @@ int tiled_variant(TiledPlan* plan);
 // Self-test of the bounded wait (an mbarrier nothing arrives at); *gave_up = 1
 // when the wait expired and raised the flag as it must.
 int tiled_wait_selftest(int* gave_up);
-// Resident CTAs per SM the kernels of a tile height are built for.
-int tiled_ctas_per_sm(int variant);
-// Allow the batch kernel of the given tile height smem_bytes of dynamic shared memory.
-int tiled_batch_prepare(int smem_bytes, int variant);
+// The tile shape of a batch's kernel: for a tile height and its highest order.
+int tiled_batch_shape(int variant, int max_N);
+// Resident CTAs per SM of that kernel with smem_bytes of dynamic shared memory.
+int tiled_batch_ctas(int smem_bytes, int shape);
+// Allow it smem_bytes of dynamic shared memory.
+int tiled_batch_prepare(int smem_bytes, int shape);
 // items: device array of int4 (instance, first tile, tile count, stride),
 // each the tiles first, first + stride, ... of one instance; CTA b runs
 // items off[b] .. off[b + 1] - 1 (off: grid + 1 device ints); params: device array
 // of 4 * instances parameter blocks (instance i, parity P, which at
 // 4 i + 2 P + which).
 int tiled_batch_pass(const void* params, const void* items, const int* off, int P, int which, int grid,
-                     int smem_bytes, int variant, void* stream);
+                     int smem_bytes, int shape, void* stream);
 
 }  // namespace starmap

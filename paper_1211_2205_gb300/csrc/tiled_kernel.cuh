@@ -1,12 +1,11 @@
 // Tiled half-step pass for the 2D real P_N system in FP32 (sm_103a).
 //
 // One CTA owns a TX x TY tile of point indices, shared by the four staggered
-// grids (section 4.1); each consumer thread owns a pair of points in each of
-// RW rows of the tile.  A
-// pass updates the components of one parity (odd l: grids G21 (R) and G12
-// (I); even l: G11 (R) and G22 (I)) from the half-grid differences
-// (eq. central_differences) of the other parity, weighted by -Mx/dx and
-// -My/dy, followed by the exact sub-step u <- a u + b (W + q)
+// grids (section 4.1); each consumer thread owns RB rows of a pair of points
+// (x, x + 1).  A pass updates the components of one parity (odd l: grids G21
+// (R) and G12 (I); even l: G11 (R) and G22 (I)) from the half-grid
+// differences (eq. central_differences) of the other parity, weighted by
+// -Mx/dx and -My/dy, followed by the exact sub-step u <- a u + b (W + q)
 // (eq. sub_step_solution).
 //
 // Streaming by moment order.  Input components of order l' are visited in
@@ -25,76 +24,93 @@
 // Every input value is read from HBM once, every output read and written
 // once; the differences of an input are formed once per point.
 //
-// Data movement: one producer warp walks a host-built stage list and issues
+// Data movement: two producer warps walk a host-built stage list and issue
 // the TMA boxes (cp.async.bulk.tensor.3d) of each stage into a ring of
 // shared-memory stages guarded by mbarriers (full: transaction bytes, empty:
 // one arrival per consumer warp).  A stage is one step of the consumer loop:
 // slots for the R and I input of (l', q') and the R and I output finalised
 // there.  Input boxes are BX x (TY+1) (one-point halo, x start aligned to 16
-// bytes); output boxes TX x TY.  Boundary conditions live in ghost cells
-// (section 4.2), which a separate refresh kernel rewrites after the pass
-// (the boundary tiles would otherwise wait on scattered single-value
-// stores).  Every wait is bounded: on expiry the kernel raises an error
-// flag, waits (bounded) for its copies in flight, and returns.
+// bytes); output boxes TX x TY.  The I input that m' = 0 does not have is a
+// box wholly outside the tensor, which TMA fills with zeros (no memory
+// traffic), so the consumers need no case for it.  Boundary conditions live
+// in ghost cells (section 4.2), which the lanes at the grid's edge write with
+// the boundary values they copy.  Every wait is bounded: on expiry the kernel raises an
+// error flag, waits (bounded) for its copies in flight, and returns.
 //
-// The file is compiled once per tile height: STARMAP_TILED_NS names the
-// namespace, STARMAP_TILED_TY the tile height, STARMAP_TILED_RW the rows per
-// consumer warp and STARMAP_TILED_MINB the CTAs per SM the launch bounds ask
-// for (10 rows, two per warp, one CTA per SM, for large N: a warp's fixed
-// cost per step (barrier wait, table reads, release) is spread over four
-// points; 5 rows, one per warp, two CTAs per SM, so that one CTA's setup,
-// fill and drain overlap the other's streaming when a tile has few stages).
+// What bounds it.  At N = 39 on 1024^2 the memory: 865 us per pass, 5.97 TB/s
+// of algorithmic traffic, 90 % of a plain copy's rate.  At low orders and on
+// grids that L2 holds, the chain of a consumer warp's steps: its instructions,
+// their latency and their fetch (two dozen steps in flight on an SM are not
+// enough to hide it).  So a step is as short as it goes:
+//   * it carries the differences of the previous input, not four accumulators
+//     (a target's sum is completed where it is finalised, in the same order
+//     of additions), so one copy of the loop body serves every step;
+//   * its branches are uniform by construction (votes, redux): no
+//     reconvergence code; boundary work is predicated stores behind one
+//     branch;
+//   * a stage's weights (each twice, as an f32x2 pair), offset and source
+//     address are one record, read before the stage's barrier;
+//   * a thread takes several adjacent rows of a pair where the warps are
+//     enough (tiled.cu): the fixed part is shared and d_y needs one load per
+//     row;
+//   * both kinds run the same code (three 4-byte loads per d_x instead of a
+//     template on the x shift): two copies missed the instruction cache.
+// Against the kernel before (four accumulators, a branch per case, a separate
+// kernel for the boundary copies, one warp issuing every box): P_13 512^2 59 ->
+// 39 us per pass, P_9 1501 x 1099 150 -> 103, N = 3 at 1024^2 35 -> 19, P_39
+// 1024^2 925 -> 862, the 16-instance batch 358 -> 224.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <utility>
 
 #include "pdl.h"
 
-#ifndef STARMAP_TILED_NS
-#define STARMAP_TILED_NS tiled
-#define STARMAP_TILED_TY 10
-#define STARMAP_TILED_MINB 1
-#define STARMAP_TILED_RW 2
-#endif
-
 namespace starmap {
-namespace STARMAP_TILED_NS {
+namespace tiled {
 
-constexpr int PX = 1;                   // point pairs per consumer thread along x
-constexpr int TX = 64 * PX;             // tile width
-constexpr int TY = STARMAP_TILED_TY;    // tile height
-constexpr int RW = STARMAP_TILED_RW;    // tile rows per consumer warp
-constexpr int RSTEP = TY / RW;          // rows between the rows of one warp
-constexpr int PP = PX * RW;             // point pairs per consumer thread: pair j of lane l covers
-                                        // x = x0 + 64 (j % PX) + 2 l, +1 in row row0 + RSTEP (j / PX)
-static_assert(TY % RW == 0, "the rows of a tile split evenly over the warps");
-constexpr int MINB = STARMAP_TILED_MINB;
+constexpr int TX = 64;                  // tile width: 32 lanes x 2 points
 constexpr int VEC = 4;                  // 16 bytes of FP32: TMA x alignment
 constexpr int BX = TX + VEC;            // input box width (halo + alignment)
-constexpr int BYI = TY + 1;             // input box height (halo)
-constexpr int IN_BYTES = BX * BYI * 4;
-constexpr int OUT_BYTES = TX * TY * 4;
-constexpr int IN_SLOT = ((IN_BYTES + 127) / 128) * 128;    // slot strides in bytes
-constexpr int OUT_SLOT = ((OUT_BYTES + 127) / 128) * 128;
-// a stage (one consumer step) holds the input R, input I, output R, output I boxes
-constexpr int STAGE_BYTES = 2 * IN_SLOT + 2 * OUT_SLOT;
-__host__ __device__ constexpr int slot_off(int slot) { return slot < 2 ? slot * IN_SLOT : 2 * IN_SLOT + (slot - 2) * OUT_SLOT; }
 constexpr int MAX_STAGES = 15;          // ring depth limit (the host fills the shared memory up to it)
-constexpr int CONSUMER_WARPS = 2 * RSTEP;   // per output kind (R, I), one warp per RW rows
-constexpr int CONSUMERS = CONSUMER_WARPS * 32;
-constexpr int PRODUCER_WARPS = 2;       // independent TMA issue streams (stage s mod 2)
-constexpr int THREADS = CONSUMERS + 32 * PRODUCER_WARPS;
+constexpr int PRODUCER_WARPS = 2;       // one issues the input boxes, one the output boxes
+
+// A tile of NB_ bands of RB_ rows, a consumer warp per band and output kind;
+// MINB_: resident CTAs per SM the registers are limited for; DUP_: each
+// weight twice in shared memory (an f32x2 pair ready to use), else once.
+template <int RB_, int NB_, int MINB_, bool DUP_>
+struct Shape {
+    static constexpr int RB = RB_, NB = NB_, MINB = MINB_;
+    static constexpr bool DUP = DUP_;
+    static constexpr int TY = RB * NB;              // tile height
+    static constexpr int BYI = TY + 1;              // input box height (halo)
+    static constexpr int IN_BYTES = BX * BYI * 4;
+    static constexpr int OUT_BYTES = TX * TY * 4;
+    static constexpr int IN_SLOT = ((IN_BYTES + 127) / 128) * 128;    // slot strides in bytes
+    static constexpr int OUT_SLOT = ((OUT_BYTES + 127) / 128) * 128;
+    // a stage (one consumer step) holds the input R, input I, output R, output I boxes
+    static constexpr int STAGE_BYTES = 2 * IN_SLOT + 2 * OUT_SLOT;
+    static constexpr int CONSUMER_WARPS = 2 * NB;   // per output kind (R, I), one warp per band
+    static constexpr int CONSUMERS = CONSUMER_WARPS * 32;
+    static constexpr int THREADS = CONSUMERS + 32 * PRODUCER_WARPS;
+    static constexpr int PART_BYTES = RB * CONSUMERS * 8;             // partial sums of one q
+    static constexpr int REC_BYTES = DUP ? 80 : 48;                   // record of a stage and kind in shared memory
+};
 constexpr int MAXN = 63;
-constexpr int RING_OFF = 256;           // full[MAX_STAGES], empty[MAX_STAGES], abort flag
-static_assert(2 * MAX_STAGES * 8 + 4 <= RING_OFF, "barriers fit before the ring");
+// Shared memory: full[MAX_STAGES], empty[MAX_STAGES], abort flag; partial
+// sums; tables; ring.  (A step may read one q past the partial sums: table
+// values that nothing uses.)
+constexpr int PART_OFF = 256;
+static_assert(2 * MAX_STAGES * 8 + 4 <= PART_OFF, "barriers fit before the partial sums");
 constexpr unsigned long long WAIT_NS = 2000000000ull;   // bounded waits: 2 s
 
 struct OutGrid {
     float* base;        // point (0,0) of component 0
     long cstride;       // elements between components
-    const float* coef;  // decay coefficients [cls][4][ny][nx]
+    const float* coef;  // decay coefficients [cls][4][ny][cp]
     int nx, ny;
+    int cp;             // row pitch of coefficients and sources (even, >= nx)
 };
 
 struct Params {
@@ -103,22 +119,23 @@ struct Params {
     long pitch;
     int p[2];
     int tiles_x;
+    int skew;                   // tile order (tile_column)
     int N, P;                   // moment order, pass parity (1 odd, 0 even)
     int which;                  // 0 half-step coefficients, 1 full-step
     int nclasses;               // 2 = isotropic (class 0: l = 0, 1: l >= 1), else class = l
-    int nstages, nin, nfin;
+    int nstages;
     int nring;                  // stages in the ring (2 .. MAX_STAGES)
     int top;                    // highest output order finalised: N, or N - 1 when every order-N
                                 // component is frozen (a closure sets them)
-    const int4* stages;         // per stage: component (in its grid) of slot 0..3, -1 if absent
-    const float4* coef[2];      // per output kind K, per q step: (cx Pm, cx P0, cx N0, cx Np) of the
-                                // input of kind K and (cy Pm, cy P0, cy N0, cy Np) of the other
-                                // input; zero if absent
-    const int2* fin[2];         // per output kind K, per finalising stage: (element offset of the
-                                // component / 32, or -1 if absent; source slot or -1)
-    const float* const* srcs;   // source arrays by slot
+    const int4* stages;         // per stage: component (in its grid) of slot 0..3, -1 if absent (an absent
+                                // I input: a component outside the tensor, a box of zeros)
+    const float4* rec[2];       // per output kind K, per stage: (P0 x, P0 y, Np x, Np y) of the previous
+                                // input of the order, (Pm x, Pm y, N0 x, N0 y) of the stage's input (x:
+                                // -Mx/dx, y: -My/dy; zero if absent), and as integers (element offset
+                                // of the target completed / 32, or -1; 0; address of its source or 0)
     int* err;                   // bounded-wait failure flag
-    int smem_coef_off[2], smem_fin_off[2], smem_part_off, smem_stage_off;   // byte offsets in dynamic smem
+    int smem_rec_off[2], smem_stage_off, smem_ring_off;     // byte offsets in dynamic smem
+    int any_src[2];             // per output kind: whether any finalised component has a source
     const float* pf_src[2];     // per output kind: the source array its finalisations read, if it
                                 // has exactly one (prefetched into L2 with the decay pairs), else null
 };
@@ -168,6 +185,22 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, i
         "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
         ::"r"(smem_u32(dst)), "l"((unsigned long long)map), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
         : "memory");
+}
+
+// The same by 32-bit shared addresses.
+__device__ __forceinline__ void expect_tx(uint32_t bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void tma_box(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+        ::"r"(dst), "l"((unsigned long long)map), "r"(x), "r"(y), "r"(z), "r"(bar)
+        : "memory");
+}
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\tselp.u32 %0, 1, 0, e;\n\t}\n" : "=r"(p));
+    return p != 0;
 }
 
 // Wait for a barrier phase with a time limit; on expiry raise the CTA's
@@ -228,38 +261,431 @@ __device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
     return d;
 }
 __device__ __forceinline__ f2 lds2(const float* p) { return *reinterpret_cast<const f2*>(p); }
+__device__ __forceinline__ f2 ldg2(const float* p) { return __ldg(reinterpret_cast<const f2*>(p)); }
 __device__ __forceinline__ f2 zero2() { return 0ull; }
 
-// float offsets of point pair j from pair 0 inside an input box / an output box
-__host__ __device__ constexpr int in_off(int j) { return (j / PX) * RSTEP * BX + 64 * (j % PX); }
-__host__ __device__ constexpr int out_off(int j) { return (j / PX) * RSTEP * TX + 64 * (j % PX); }
 
-// x-differences of points A (column c) and B (column c + 1) of one box row:
-// right operands at columns c, c + 1, left operands at c - 1, c.  The pair
-// load starts at the even column of the two.
-__device__ __forceinline__ f2 diff_x(const float* row, int c, bool c_even) {
-    if (c_even) {
-        const f2 P = lds2(row + c);                 // v[c], v[c+1]
-        const float Q = row[c - 1];
-        float lo, hi;
-        f2_split(P, lo, hi);
-        return f2_sub(P, f2_make(Q, lo));
+// The source address of a finalise entry.
+__device__ __forceinline__ const float* source_of(const int4& f) {
+    return reinterpret_cast<const float*>(((unsigned long long)(unsigned)f.w << 32) | (unsigned)f.z);
+}
+
+// Slots of a stage: byte offsets of the R / I input boxes and the R / I output boxes.
+template <class S>
+__host__ __device__ constexpr int slot_off(int slot) {
+    return slot < 2 ? slot * S::IN_SLOT : 2 * S::IN_SLOT + (slot - 2) * S::OUT_SLOT;
+}
+
+// The weighted differences of one q step for a pair of points: x and y hold
+// the weights of the targets Pm, P0, N0, Np for d_x and d_y.  Nn starts here
+// (Np is the first contribution to its target from this order).
+__device__ __forceinline__ void add_targets(f2 dx, f2 dy, const f2 (&x)[4], const f2 (&y)[4], f2& Pc, f2& Pn, f2& Nc,
+                                            f2& Nn) {
+    Pc = f2_fma(x[0], dx, Pc);
+    Pn = f2_fma(x[1], dx, Pn);
+    Nc = f2_fma(x[2], dx, Nc);
+    Nn = f2_fma(x[3], dx, zero2());
+    Pc = f2_fma(y[0], dy, Pc);
+    Pn = f2_fma(y[1], dy, Pn);
+    Nc = f2_fma(y[2], dy, Nc);
+    Nn = f2_fma(y[3], dy, Nn);
+}
+
+// The weights of a step (cp[0]: x, cp[1]: y), each as an f32x2 pair.
+__device__ __forceinline__ void load_weights(const float4* cp, f2 (&x)[4], f2 (&y)[4]) {
+    const float4 a = cp[0], b = cp[1];
+    x[0] = f2_make(a.x, a.x); x[1] = f2_make(a.y, a.y); x[2] = f2_make(a.z, a.z); x[3] = f2_make(a.w, a.w);
+    y[0] = f2_make(b.x, b.x); y[1] = f2_make(b.y, b.y); y[2] = f2_make(b.z, b.z); y[3] = f2_make(b.w, b.w);
+}
+
+// Shared memory by 32-bit address (the consumers' inner loop).
+template <int OFF>
+__device__ __forceinline__ f2 ld8(uint32_t a) {
+    f2 v;
+    asm volatile("ld.shared.b64 %0, [%1+%2];" : "=l"(v) : "r"(a), "n"(OFF));
+    return v;
+}
+template <int OFF>
+__device__ __forceinline__ float ld4(uint32_t a) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1+%2];" : "=f"(v) : "r"(a), "n"(OFF));
+    return v;
+}
+template <int OFF>
+__device__ __forceinline__ void ld16(uint32_t a, f2& x, f2& y) {
+    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2+%3];" : "=l"(x), "=l"(y) : "r"(a), "n"(OFF));
+}
+__device__ __forceinline__ int4 ld16i(uint32_t a) {
+    int4 v;
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+    return v;
+}
+template <int OFF>
+__device__ __forceinline__ void st8(uint32_t a, f2 v) {
+    asm volatile("st.shared.b64 [%0+%1], %2;" ::"r"(a), "n"(OFF), "l"(v));
+}
+// The four weights of one half of a stage record, as f32x2 pairs.
+template <bool DUP, int HALF>
+__device__ __forceinline__ void ld_weights(uint32_t a, f2 (&w)[4]) {
+    if constexpr (DUP) {
+        ld16<32 * HALF>(a, w[0], w[1]);
+        ld16<32 * HALF + 16>(a, w[2], w[3]);
+    } else {
+        f2 p[2];
+        ld16<16 * HALF>(a, p[0], p[1]);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            float u, v;
+            f2_split(p[i], u, v);
+            w[2 * i] = f2_make(u, u);
+            w[2 * i + 1] = f2_make(v, v);
+        }
     }
-    const f2 P = lds2(row + c - 1);                 // v[c-1], v[c]
-    const float Q = row[c + 1];
-    float lo, hi;
-    f2_split(P, lo, hi);
-    return f2_sub(f2_make(hi, Q), P);
+}
+
+// A value every lane holds, as the compiler can see (the batch reads its
+// parameters from shared memory): branches on it need no reconvergence.
+__device__ __forceinline__ int uni(int v) { return __reduce_max_sync(0xffffffffu, v); }
+
+// wait_bounded for a whole warp: all lanes take part and leave together.
+__device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err) {
+    auto test = [&]() -> bool {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}\n"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        return __all_sync(0xffffffffu, ok != 0);
+    };
+    if (test()) return true;
+    const unsigned long long t0 = global_ns();
+    while (!test()) {
+        if (__any_sync(0xffffffffu, *abort_flag != 0)) return false;
+        if (__any_sync(0xffffffffu, global_ns() - t0 > WAIT_NS)) {
+            *abort_flag = 1;
+            atomicExch(err, 1);
+            return false;
+        }
+    }
+    return true;
+}
+// One arrival of the warp (all lanes' reads before it).
+__device__ __forceinline__ void arrive_warp(uint32_t bar, int lane) {
+    __syncwarp();
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.s32 p, %1, 0;\n\t@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}\n" ::"r"(bar),
+                 "r"(lane)
+                 : "memory");
+}
+
+// Global stores of the lanes with i < n (predicated: as branches they cost
+// more than the stores).
+template <int I>
+__device__ __forceinline__ void st8_if(float* p, f2 v, int n) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.gt.s32 p, %2, %3;\n\t@p st.global.b64 [%0], %1;\n\t}\n" ::"l"(p), "l"(v), "r"(n), "n"(I));
+}
+template <int I>
+__device__ __forceinline__ void st4_if(float* p, float v, int n) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.gt.s32 p, %2, %3;\n\t@p st.global.f32 [%0], %1;\n\t}\n" ::"l"(p), "f"(v), "r"(n), "n"(I));
+}
+
+// v, with its origin hidden: what is computed from it is not hoisted out of
+// the loops, where it would hold registers.
+__device__ __forceinline__ int here(int v) { asm volatile("" : "+r"(v)); return v; }
+__device__ __forceinline__ long here(long v) { asm volatile("" : "+l"(v)); return v; }
+
+// f(row) for the rows of a thread, the row a compile-time constant (an immediate offset).
+template <class F, int... I>
+__device__ __forceinline__ void each_row(F&& f, std::integer_sequence<int, I...>) {
+    (f(std::integral_constant<int, I>{}), ...);
+}
+
+// Column of tile `tile` in row `row`: in raster order, or (skew) each row
+// starting one column further than the row before, so that a CTA's strided
+// run of tiles does not stay in one column (the edge columns cost more).
+__device__ __forceinline__ int tile_column(const Params& prm, int tile, int row) {
+    int c = tile - row * prm.tiles_x;
+    if (prm.skew) c = (c + row) % prm.tiles_x;
+    return c;
+}
+
+// Consumer warps of one CTA: the tiles t0, t0 + tstride, ... (ntl of them).
+// Warp w handles rows RB band .. RB band + RB - 1 (band = w % NB) of the tile
+// for the targets of kind K = w / NB (0: R outputs, 1: I outputs), lane l the
+// points A = x0 + 2 l and B = A + 1.  Targets of kind K take d_x of the
+// inputs of kind K (slot K, through Mx) and d_y of the other kind's (slot
+// 1 - K, through My).  sxK, syK: shifts of the right / upper operand of kind
+// K's input (input_shift).
+//
+// Step q of order lp has the differences of input (lp, q) at hand and, in
+// registers, those of input (lp, q - 1); it completes the previous-order
+// target (lp - 1, q - 1) (partial sum, then input q - 1, then input q) and
+// what order lp adds to the next-order target (lp + 1, q).
+template <class S>
+__device__ __forceinline__ void consume(const Params& prm, int K, int sxK, int syK, int t0, int tstride, int ntl) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    constexpr int RB = S::RB;
+    constexpr auto ROWS = std::make_integer_sequence<int, RB>{};
+    constexpr int PI = S::CONSUMERS * 8;                // bytes between a thread's partial sums of two rows
+    constexpr int PQ = RB * PI;                         // and of two q
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + 2 * MAX_STAGES * 8);
+    const uint32_t base = smem_u32(smem);
+    const uint32_t ring = base + prm.smem_ring_off;
+    const int NR = uni(prm.nring);
+    const int tid = threadIdx.x;
+    const int lane = tid & 31, band = (tid >> 5) % S::NB;
+    const uint32_t part = base + PART_OFF + 8 * tid;    // entry (q, i) at part + q PQ + i PI
+    // byte offsets inside a stage, row i of the thread at + 4 i BX (+ 4 i TX):
+    // the aligned pair and the single value of d_x, the lower operands of
+    // d_y (both boxes start one row below the first row that is read from
+    // below, so d_y always takes box rows r and r + 1), the old value
+    const int ox = slot_off<S>(K) + 4 * ((RB * band + (syK == 0 ? 1 : 0)) * BX + 2 * lane + (sxK == 0 ? VEC - 1 : 0));
+    const int oy = slot_off<S>(1 - K) + 4 * (RB * band * BX + 2 * lane + (sxK == 0 ? 0 : VEC));
+    const int ou = slot_off<S>(2 + K) + 4 * (RB * band * TX + 2 * lane);
+    const OutGrid& G = prm.out[K];
+    const int N = uni(prm.N), first = 1 - uni(prm.P);   // first input order: even l' for the odd pass
+    const int top = uni(prm.top), ncls = uni(prm.nclasses);
+    const bool any_src = uni(prm.any_src[K]) != 0;
+    // whether an axis of the output grid keeps copies (section 4.2: every axis but an extrapolation axis
+    // of nodes); periodic -1 <- n - 1, n <- 0; extrapolation -1 <- 0, n <- n - 1; corners by both rules
+    const int px = prm.p[0], py = prm.p[1];
+    const bool hx = px || (prm.P == 1) == (K == 1), hy = py || K == 0;
+    int r = 0;                                          // ring slot and phase of the next stage
+    uint32_t ph = 0;
+    int done = 0;                                       // stages consumed
+    for (int tl = 0; tl < ntl; ++tl) {
+        const int tile = t0 + tl * tstride;
+        const int trow = tile / prm.tiles_x;
+        const int gx = tile_column(prm, tile, trow) * TX + 2 * lane;
+        const int gy = trow * S::TY + RB * band;
+        // rows in which the lane stores both points, or A alone (the last column of an odd width)
+        const int nrow = max(0, min(RB, G.ny - gy));
+        const int both = gx + 1 < G.nx ? nrow : 0, lone = gx + 1 == G.nx ? nrow : 0;
+        // ghost-cell copies of the warp's points: along x the lane's copy of A (or B: cb) lands xo
+        // elements from A in xrow rows (xo2: a second one, in a grid narrower than three); along y row il
+        // of the warp is copied to row -1 and row ir to row ny (-1: neither)
+        int xo = 0, xo2 = 0;
+        bool cb = false;
+        if (hx) {
+            const int xl = px ? G.nx - 1 : 0, xr = px ? 0 : G.nx - 1;
+            const bool l = xl == gx || xl == gx + 1, r = xr == gx || xr == gx + 1;
+            xo = l ? -1 - gx : r ? G.nx - gx : 0;
+            cb = (l ? xl : xr) != gx;
+            if (l && r) xo2 = G.nx - gx;
+        }
+        const int xrow = xo != 0 ? nrow : 0;
+        int il = -1, ir = -1;
+        if (hy) {
+            il = (py ? G.ny - 1 : 0) - gy;
+            ir = (py ? 0 : G.ny - 1) - gy;
+            if (il < 0 || il >= RB) il = -1;
+            if (ir < 0 || ir >= RB) ir = -1;
+        }
+        il = uni(il);
+        ir = uni(ir);
+        const bool tiny = __any_sync(0xffffffffu, xo2 != 0);
+        const bool edge = __any_sync(0xffffffffu, lone != 0 || xrow != 0 || tiny || il >= 0 || ir >= 0);
+        float* const dst0 = G.base + (long)(gy + 1) * prm.pitch + gx;   // point A of row 0 in component 0
+        // coefficient / source index of point A of row 0, and the last row's offset in rows; points
+        // outside the grid read a valid place and are never stored
+        const long c0 = (long)min(gy, G.ny - 1) * G.cp + min(gx, G.cp - 2);
+        const int cmax = max(G.ny - 1 - gy, 0);
+        uint32_t rec = base + prm.smem_rec_off[K];      // the stage's record
+        int cls = -1;
+        f2 aL[RB], bL[RB];                              // decay pairs (a, b) of the outputs being finalised
+        f2 W[RB];                                       // sum of the target being completed
+        // the stage's barrier and its release
+        auto wait = [&]() -> bool { return wait_warp(base + 8 * r, ph, abort_flag, prm.err); };
+        auto release = [&]() {
+            arrive_warp(base + 8 * (MAX_STAGES + r), lane);
+            ++done;
+            if (++r == NR) { r = 0; ph ^= 1u; }
+        };
+        // differences of the stage's input
+        auto differences = [&](uint32_t t, f2 (&dx)[RB], f2 (&dy)[RB]) {
+            const uint32_t tx = t + ox, ty = t + oy;
+            f2 lo = ld8<0>(ty);
+            each_row([&](auto i) {
+                const f2 hi = ld8<4 * (i + 1) * BX>(ty);
+                dy[i] = f2_sub(hi, lo);
+                lo = hi;
+                const float a = ld4<4 * i * BX>(tx), b = ld4<4 * i * BX + 4>(tx), c = ld4<4 * i * BX + 8>(tx);
+                dx[i] = f2_make(b - a, c - b);
+            }, ROWS);
+        };
+        // row `row` of v to the ghost row whose point A is at g, with its own copies along x
+        auto copy_row = [&](f2 c, const f2 (&v)[RB], int row, float* g) {
+            each_row([&](auto i) { if (row == i) c = v[i]; }, ROWS);
+            float c0, c1;
+            f2_split(c, c0, c1);
+            st8_if<0>(g, c, both);
+            st4_if<0>(g, c0, lone);
+            st4_if<0>(g + xo, cb ? c1 : c0, xrow);
+            if (tiny && xo2 != 0) g[xo2] = (px ? 0 : G.nx - 1) == gx ? c0 : c1;
+        };
+        // u <- a u + b (W + q) of the target whose sum is W; f: its offset and source
+        auto finalise = [&](const int4& f, const f2 (&u)[RB]) {
+            if (any_src) {
+                if (__any_sync(0xffffffffu, (f.z | f.w) != 0)) {
+                    const float* sp = source_of(f) + c0;
+                    const int cm = here(cmax);
+#pragma unroll
+                    for (int i = 0; i < RB; ++i) W[i] = f2_add(W[i], ldg2(sp + min(i, cm) * G.cp));
+                }
+            }
+            float* dst = dst0 + 32 * (long)f.x;         // 64-bit: states beyond 2^31 values
+            const long pitch = here(prm.pitch);
+            f2 v[RB];
+#pragma unroll
+            for (int i = 0; i < RB; ++i) v[i] = f2_fma(aL[i], u[i], f2_mul(bL[i], W[i]));
+            float* d = dst;
+            each_row([&](auto i) { st8_if<i>(d, v[i], both); d += pitch; }, ROWS);
+            if (edge) {
+                d = dst;
+                each_row([&](auto i) {
+                    float v0, v1;
+                    f2_split(v[i], v0, v1);
+                    st4_if<i>(d, v0, lone);
+                    st4_if<i>(d + xo, cb ? v1 : v0, xrow);
+                    d += pitch;
+                }, ROWS);
+                if (tiny && xo2 != 0) {
+                    d = dst;
+                    for (int i = 0; i < RB; ++i, d += pitch) {
+                        float v0, v1;
+                        f2_split(v[i], v0, v1);
+                        if (i < nrow) d[xo2] = (px ? 0 : G.nx - 1) == gx ? v0 : v1;
+                    }
+                }
+                if (il >= 0) copy_row(v[0], v, il, dst - (long)(gy + 1) * pitch);
+                if (ir >= 0) copy_row(v[0], v, ir, dst + (long)(G.ny - gy) * pitch);
+            }
+        };
+        // a step with an input and a target to complete: differences of the
+        // previous input in, of this one out in (dx, dy)
+        auto full_step = [&](uint32_t pq, f2 (&dx)[RB], f2 (&dy)[RB]) -> bool {
+            f2 w[4], Nn[RB], u[RB];
+            ld_weights<S::DUP, 0>(rec, w);              // P0 and Np of the previous input
+#pragma unroll
+            for (int i = 0; i < RB; ++i) {
+                W[i] = f2_fma(w[0], dx[i], W[i]);
+                Nn[i] = f2_fma(w[2], dx[i], zero2());
+                W[i] = f2_fma(w[1], dy[i], W[i]);
+                Nn[i] = f2_fma(w[3], dy[i], Nn[i]);
+            }
+            ld_weights<S::DUP, 1>(rec, w);              // Pm and N0 of this input
+            const int4 f = ld16i(rec + S::REC_BYTES - 16);
+            rec += S::REC_BYTES;
+            if (!wait()) return false;
+            const uint32_t t = ring + r * S::STAGE_BYTES;
+            differences(t, dx, dy);
+            each_row([&](auto i) { u[i] = ld8<4 * i * TX>(t + ou); }, ROWS);
+            release();
+#pragma unroll
+            for (int i = 0; i < RB; ++i) {
+                W[i] = f2_fma(w[0], dx[i], W[i]);
+                Nn[i] = f2_fma(w[2], dx[i], Nn[i]);
+                W[i] = f2_fma(w[1], dy[i], W[i]);
+                Nn[i] = f2_fma(w[3], dy[i], Nn[i]);
+            }
+            finalise(f, u);
+            each_row([&](auto i) {
+                W[i] = ld8<i * PI>(pq);
+                st8<i * PI>(pq, Nn[i]);
+            }, ROWS);
+            return true;
+        };
+        if (first == 1)                         // the even pass completes order 0 after order 1 alone: no partial sums yet
+            each_row([&](auto i) { st8<i * PI>(part, zero2()); }, ROWS);
+        // input orders, then (lp > N) the outputs of the order above the last input order
+        for (int lp = first;; lp += 2) {
+            const bool body = lp <= N;
+            if (!body && lp - 1 > top) break;
+            const int want = ncls == 2 ? min(lp - 1, 1) : lp - 1;
+            if (want >= 0 && want != cls) {
+                // used one step later at the earliest (or at once in the last order)
+                cls = want;
+                const long plane = here((long)G.cp * G.ny);
+                const int cm = here(cmax);
+                const float* ca = G.coef + ((long)cls * 4 + 2 * prm.which) * plane + c0;
+                const float* cb = ca + plane;
+#pragma unroll
+                for (int i = 0; i < RB; ++i) aL[i] = ldg2(ca + min(i, cm) * G.cp);
+#pragma unroll
+                for (int i = 0; i < RB; ++i) bL[i] = ldg2(cb + min(i, cm) * G.cp);
+            }
+            uint32_t pq = part;                 // partial sums of the step
+            int left;                           // steps that only complete a target
+            f2 dx[RB], dy[RB];
+            if (body) {
+                // q = 0: no target of order lp - 1 to complete yet
+                f2 w[4], Nn[RB];
+                ld_weights<S::DUP, 1>(rec, w);
+                rec += S::REC_BYTES;
+                if (!wait()) return;
+                differences(ring + r * S::STAGE_BYTES, dx, dy);
+                release();
+                each_row([&](auto i) {
+                    Nn[i] = f2_fma(w[3], dy[i], f2_fma(w[2], dx[i], zero2()));
+                    W[i] = ld8<i * PI>(pq);
+                    st8<i * PI>(pq, Nn[i]);
+                }, ROWS);
+                for (int q = nq_of(lp) - 1; q > 0; --q) {
+                    pq += PQ;
+                    if (!full_step(pq, dx, dy)) return;
+                }
+                left = lp & 1;                  // an odd order's last target has no further input
+            } else {
+                left = nq_of(lp - 1);
+#pragma unroll
+                for (int i = 0; i < RB; ++i) dx[i] = dy[i] = zero2();
+                each_row([&](auto i) { W[i] = ld8<i * PI>(pq); }, ROWS);
+            }
+            for (; left > 0; --left) {
+                f2 w[4], Nn[RB], u[RB];
+                ld_weights<S::DUP, 0>(rec, w);
+#pragma unroll
+                for (int i = 0; i < RB; ++i) {
+                    W[i] = f2_fma(w[0], dx[i], W[i]);
+                    Nn[i] = f2_fma(w[2], dx[i], zero2());
+                    W[i] = f2_fma(w[1], dy[i], W[i]);
+                    Nn[i] = f2_fma(w[3], dy[i], Nn[i]);
+                }
+                const int4 f = ld16i(rec + S::REC_BYTES - 16);
+                rec += S::REC_BYTES;
+                if (!wait()) return;
+                const uint32_t t = ring + r * S::STAGE_BYTES;
+                each_row([&](auto i) { u[i] = ld8<4 * i * TX>(t + ou); }, ROWS);
+                release();
+                if (__any_sync(0xffffffffu, f.x >= 0)) finalise(f, u);
+                pq += PQ;
+                if (body) {
+                    if (lp < N) each_row([&](auto i) { st8<i * PI>(pq, Nn[i]); }, ROWS);
+                } else {
+                    each_row([&](auto i) { W[i] = ld8<i * PI>(pq); }, ROWS);
+                }
+            }
+            if (!body) break;
+        }
+        // every tile consumes exactly the stages the producers issue for it
+        if (done != (tl + 1) * prm.nstages) {
+            atomicExch(prm.err, 1);
+            return;
+        }
+    }
 }
 
 // Tiles t0, t0 + tstride, ... < tend of one pass, through one continuous
-// pipeline: the producers walk a global stage index over all of them (the
+// pipeline: the producer walks a global stage index over all of them (the
 // first stages of the next tile are in flight while the consumers finish
 // the current one), the consumers step through the tiles in the same order.
 // maps: the pass's four tensor maps (in parameter or global memory: TMA
 // reads them from there); prm: everything else.  first_call: the CTA's
 // first call (a later call invalidates and re-initialises the barriers; the
 // caller synchronises the CTA in between).
+template <class S>
 __device__ __forceinline__ void tiled_tiles(const Params& prm, const CUtensorMap* maps, int t0, int tstride, int tend,
                                             bool first_call) {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -267,16 +693,14 @@ __device__ __forceinline__ void tiled_tiles(const Params& prm, const CUtensorMap
     uint64_t* empty = full + MAX_STAGES;
     volatile int* abort_flag = reinterpret_cast<volatile int*>(empty + MAX_STAGES);
     const int NR = prm.nring;
-    unsigned char* ring = smem + RING_OFF;
-    f2* s_part = reinterpret_cast<f2*>(smem + prm.smem_part_off);
-    const int4* s_stages = reinterpret_cast<const int4*>(smem + prm.smem_stage_off);
+    const uint32_t base = smem_u32(smem), ring = base + prm.smem_ring_off;
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5, lane = tid & 31;
     const int ntl = t0 < tend ? (tend - t0 + tstride - 1) / tstride : 0;
 
     // warm the TMA descriptor cache while the barriers and tables are set up
-    if (warp == CONSUMER_WARPS && lane < 4)
+    if (warp == S::CONSUMER_WARPS && lane < 4)
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(maps + lane)) : "memory");
     if (tid == 0) {
         for (int r = 0; r < MAX_STAGES; ++r) {      // every barrier: a batch's items differ in depth
@@ -284,22 +708,30 @@ __device__ __forceinline__ void tiled_tiles(const Params& prm, const CUtensorMap
                 mbar_inval(&full[r]);
                 mbar_inval(&empty[r]);
             }
-            mbar_init(&full[r], 1);
-            mbar_init(&empty[r], CONSUMER_WARPS);
+            mbar_init(&full[r], PRODUCER_WARPS);
+            mbar_init(&empty[r], S::CONSUMER_WARPS);
         }
         *abort_flag = 0;
         fence_mbar_init();
     }
-    // stage the coefficient, finalise and stage tables in shared memory
+    // stage the records and the stage list in shared memory
     for (int k = 0; k < 2; ++k) {
-        float4* c = reinterpret_cast<float4*>(smem + prm.smem_coef_off[k]);
-        for (int i = tid; i < 2 * prm.nin; i += THREADS) c[i] = __ldg(prm.coef[k] + i);
-        int2* f = reinterpret_cast<int2*>(smem + prm.smem_fin_off[k]);
-        for (int i = tid; i < prm.nfin; i += THREADS) f[i] = __ldg(prm.fin[k] + i);
+        unsigned char* rec = smem + prm.smem_rec_off[k];
+        for (int i = tid; i < 3 * prm.nstages; i += S::THREADS) {
+            const float4 w = __ldg(prm.rec[k] + i);
+            const int stage = i / 3, part = i % 3;
+            float4* d = reinterpret_cast<float4*>(rec + stage * S::REC_BYTES);
+            if (!S::DUP || part == 2) {
+                d[S::DUP ? 4 : part] = w;
+            } else {
+                d[2 * part] = make_float4(w.x, w.x, w.y, w.y);
+                d[2 * part + 1] = make_float4(w.z, w.z, w.w, w.w);
+            }
+        }
     }
     {
         int4* st = reinterpret_cast<int4*>(smem + prm.smem_stage_off);
-        for (int i = tid; i < prm.nstages; i += THREADS) st[i] = __ldg(prm.stages + i);
+        for (int i = tid; i < prm.nstages; i += S::THREADS) st[i] = __ldg(prm.stages + i);
     }
     __syncthreads();
     if (first_call) {
@@ -313,310 +745,83 @@ __device__ __forceinline__ void tiled_tiles(const Params& prm, const CUtensorMap
     input_shift(prm.P, 0, prm.p[0], prm.p[1], sxR, syR);
     input_shift(prm.P, 1, prm.p[0], prm.p[1], sxI, syI);
 
-    // --------------------------------------------------------- producer
-    // Producer warp pw owns the global stages G = pw (mod PRODUCER_WARPS)
-    // over all of the CTA's tiles (stage k of tile t is G = t * nstages + k,
-    // ring slot G mod nring).  Lane 0 waits for the slot to drain and arms
-    // its barrier with the byte count; lanes 0..3 then issue the (up to) four
-    // boxes, lane = slot.
-    if (warp >= CONSUMER_WARPS) {
-        const int pw = warp - CONSUMER_WARPS;
-        const int slot = lane & 3;
-        const CUtensorMap* map = maps + slot;
-        const int nst = prm.nstages;
-        const int total = ntl * nst;        // the host keeps this below 2^31
-        int last = -1;
-        bool ok = true;
-        // G = pw, pw + PRODUCER_WARPS, ...: stage k of local tile tl, ring
-        // slot r, ring round u (all advanced incrementally)
-        int k = pw, tl = 0, r = pw, u = 0;
-        while (k >= nst && nst > 0) { k -= nst; ++tl; }
-        int tile_at = -1, bx = 0, by = 0;
-        bool entered = false;   // this warp has just issued its first stage of tile tl
-        for (int G = pw; G < total; G += PRODUCER_WARPS) {
-            entered = tl != tile_at;
-            if (tl != tile_at) {
-                // box origin of this lane's slot in tile tl (tensor coordinates x' = x + VEC, row = y + 1)
-                tile_at = tl;
-                const int tile = t0 + tl * tstride;
-                const int x0 = (tile % prm.tiles_x) * TX, y0 = (tile / prm.tiles_x) * TY;
-                const int bxR = x0 + (sxR == 0 ? 0 : VEC), byR = y0 + (syR == 0 ? -1 : 0) + 1;
-                const int bxI = x0 + (sxI == 0 ? 0 : VEC), byI = y0 + (syI == 0 ? -1 : 0) + 1;
-                bx = slot == 0 ? bxR : slot == 1 ? bxI : x0 + VEC;
-                by = slot == 0 ? byR : slot == 1 ? byI : y0 + 1;
-            }
-            int4 st = make_int4(-1, -1, -1, -1);
-            if (lane < 4) st = s_stages[k];
-            const int comp = slot == 0 ? st.x : slot == 1 ? st.y : slot == 2 ? st.z : st.w;
-            const uint32_t mine = lane < 4 && comp >= 0 ? (slot < 2 ? IN_BYTES : OUT_BYTES) : 0u;
-            uint32_t bytes = mine;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) bytes += __shfl_xor_sync(0xffffffffu, bytes, o);
-            if (lane == 0) {
-                if (u > 0 && !wait_bounded(&empty[r], (u - 1) & 1, abort_flag, prm.err)) ok = false;
-                if (ok) mbar_expect_tx(&full[r], bytes);
-            }
-            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-            if (!ok) break;
-            if (mine != 0u) tma_load_3d(ring + r * STAGE_BYTES + slot_off(slot), map, bx, by, comp, &full[r]);
-            if (entered && tl > 0 && pw == 0 && prm.nclasses == 2) {
-                // the decay pairs (and the source) of this tile (not the first: there
-                // the consumers load them at once) into L2 while the consumers finish
-                // the previous tiles; lane = (kind, class, plane a / b, half row of 32)
-                const int tile = t0 + tl * tstride;
-                const int x0 = (tile % prm.tiles_x) * TX, y0 = (tile / prm.tiles_x) * TY;
-                const int kind = lane >> 4, c = (lane >> 3) & 1, ab = (lane >> 2) & 1, hx = lane & 1;
-                const OutGrid& Gk = prm.out[kind];
-                const int x = x0 + 32 * hx;
-                if (x < Gk.nx) {
-                    const long plane = (long)Gk.nx * Gk.ny;
-                    // lanes with bit 1 clear: decay pairs; lanes 2 + 16 kind (+1): the kind's source
-                    const float* base = ((lane >> 1) & 1) == 0
-                        ? (Gk.coef != nullptr ? Gk.coef + ((long)c * 4 + 2 * prm.which + ab) * plane + x : nullptr)
-                        : ((lane & 12) == 0 && prm.pf_src[kind] != nullptr ? prm.pf_src[kind] + x : nullptr);
-                    if (base != nullptr)
-                        for (int y = y0; y < y0 + TY && y < Gk.ny; ++y)
-                            asm volatile("prefetch.global.L2 [%0];" ::"l"(base + (long)y * Gk.nx));
-                }
-            }
-            last = G;
-            k += PRODUCER_WARPS;
-            while (k >= nst) { k -= nst; ++tl; }
-            r += PRODUCER_WARPS;
-            if (r >= NR) { r -= NR; ++u; }
-        }
-        if (!ok && lane == 0) {
-            // aborted: wait (bounded) for this warp's copies still in flight
-            for (int G = last; G >= 0 && G > last - NR; G -= PRODUCER_WARPS) {
-                const unsigned long long tw = global_ns();
-                while (!mbar_try_wait(&full[G % NR], (G / NR) & 1))
-                    if (global_ns() - tw > WAIT_NS) break;
-            }
-        }
+    if (warp < S::CONSUMER_WARPS) {
+        const int K = warp / S::NB;
+        const int syK = K == 0 ? syR : syI;
+        // (the two kinds' inputs lie on opposite x grids: sxI = 1 - sxR)
+        consume<S>(prm, K, K == 0 ? sxR : sxI, syK, t0, tstride, ntl);
         return;
     }
 
-    // --------------------------------------------------------- consumers
-    // Warp w handles the tile rows row0 + RSTEP i (row0 = w % RSTEP, i < RW)
-    // for the targets of kind K = w / RSTEP (0: R outputs, 1: I outputs), at
-    // the point pairs j = 0..PP-1: A_j = (x0 + 64 (j % PX) + 2 lane,
-    // y0 + row0 + RSTEP (j / PX)), B_j = A_j + (1, 0).  Targets of kind K
-    // take d_x of the inputs of kind K (through Mx) and d_y of the inputs of
-    // the other kind (through My).
-    const int K = warp / RSTEP;
-    const int row = warp % RSTEP;
-    int s = 0;                  // global consumer step (= stage) over the CTA's tiles
-    int ring_r = 0;             // its ring slot and barrier phase
-    uint32_t ring_ph = 0;
-    bool alive = true;
-    // the output grid of kind K
-    const OutGrid& G = prm.out[K];
-    const long plane = (long)G.nx * G.ny;
-    for (int tl = 0; tl < ntl && alive; ++tl) {
+    // --------------------------------------------------------- producers
+    // Producer warp h issues the two input boxes (h = 0) or the two output
+    // boxes (h = 1) of every stage of the CTA's tiles (stage k of local tile
+    // tl in ring slot r, ring round u): it waits for the slot to drain, arms
+    // its share of the slot's byte count and issues the boxes.  (With one
+    // warp for all four boxes a stage took about 800 cycles to issue, which
+    // set the pace of every pass.)
+    const int h = warp - S::CONSUMER_WARPS;
+    const int2* s_comp = reinterpret_cast<const int2*>(smem + prm.smem_stage_off) + h;
+    const CUtensorMap* mR = maps + 2 * h;
+    const CUtensorMap* mI = maps + 2 * h + 1;
+    const uint32_t box_bytes = h == 0 ? S::IN_BYTES : S::OUT_BYTES;
+    const int oR = slot_off<S>(2 * h), oI = slot_off<S>(2 * h + 1);
+    const int nst = prm.nstages;
+    int r = 0, u = 0, issued = 0;
+    bool ok = true;
+    for (int tl = 0; tl < ntl && ok; ++tl) {
+        // box origins (tensor coordinates x' = x + VEC, row = y + 1)
         const int tile = t0 + tl * tstride;
-        const int x0 = (tile % prm.tiles_x) * TX, y0 = (tile / prm.tiles_x) * TY;
-        // float offsets, inside a step, of the difference operands of pair 0
-        // (pair j sits in_off(j) floats further): d_x from the input of kind K (slot
-        // K), d_y from the input of kind 1 - K (slot 1 - K)
-        int rx, cx, uy;
-        bool ev;
-        {
-            const int sxK = K == 0 ? sxR : sxI;
-            const int syO = K == 0 ? syI : syR;
-            const int syK = K == 0 ? syR : syI;
-            const int sxO = K == 0 ? sxI : sxR;
-            const int bxsK = sxK == 0 ? -VEC : 0, oyK = syK == 0 ? -1 : 0;
-            const int bxsO = sxO == 0 ? -VEC : 0, oyO = syO == 0 ? -1 : 0;
-            rx = slot_off(K) / 4 + (row - oyK) * BX;
-            cx = 2 * lane + sxK - bxsK;
-            ev = (cx & 1) == 0;
-            uy = slot_off(1 - K) / 4 + (row + syO - oyO) * BX + (2 * lane - bxsO);
-        }
-        bool inA[PP], inB[PP], pair[PP];
-        float* pptr[PP];          // point A_j in component 0
-        long cidxA[PP];
-        f2 ca2[PP][2], cb2[PP][2];  // decay pairs by class (isotropic)
-    #pragma unroll
-        for (int j = 0; j < PP; ++j) {
-            const int gx = x0 + 64 * (j % PX) + 2 * lane;
-            const int gy = y0 + row + RSTEP * (j / PX);
-            inA[j] = gx < G.nx && gy < G.ny;
-            inB[j] = gx + 1 < G.nx && gy < G.ny;
-            pptr[j] = G.base + (long)(gy + 1) * prm.pitch + gx;
-            cidxA[j] = (long)gy * G.nx + gx;
-            pair[j] = inA[j] && inB[j];
-            for (int c = 0; c < 2; ++c) {
-                float a[2] = {0.f, 0.f}, b[2] = {0.f, 0.f};
-                if (prm.nclasses == 2 && G.coef != nullptr) {
-                    const float* cf = G.coef + (long)c * 4 * plane + cidxA[j];
-                    if (inA[j]) { a[0] = __ldg(cf + 2 * prm.which * plane); b[0] = __ldg(cf + (2 * prm.which + 1) * plane); }
-                    if (inB[j]) { a[1] = __ldg(cf + 2 * prm.which * plane + 1); b[1] = __ldg(cf + (2 * prm.which + 1) * plane + 1); }
+        const int trow = tile / prm.tiles_x;
+        const int x0 = tile_column(prm, tile, trow) * TX, y0 = trow * S::TY;
+        const int bxR = h == 0 ? x0 + (sxR == 0 ? 0 : VEC) : x0 + VEC, byR = h == 0 ? y0 + (syR == 0 ? 0 : 1) : y0 + 1;
+        const int bxI = h == 0 ? x0 + (sxI == 0 ? 0 : VEC) : x0 + VEC, byI = h == 0 ? y0 + (syI == 0 ? 0 : 1) : y0 + 1;
+        int k = 0;
+        auto issue = [&](int kend) {
+            for (; k < kend && ok; ++k) {
+                const int2 c = s_comp[2 * k];
+                if (u > 0 && !wait_warp(base + 8 * (MAX_STAGES + r), (u - 1) & 1, abort_flag, prm.err)) {
+                    ok = false;
+                    break;
                 }
-                ca2[j][c] = f2_make(a[0], a[1]);
-                cb2[j][c] = f2_make(b[0], b[1]);
+                const uint32_t dst = ring + r * S::STAGE_BYTES, bar = base + 8 * r;
+                if (elect_one()) {
+                    expect_tx(bar, ((c.x >= 0 ? 1u : 0u) + (c.y >= 0 ? 1u : 0u)) * box_bytes);
+                    if (c.x >= 0) tma_box(dst + oR, mR, bxR, byR, c.x, bar);
+                    if (c.y >= 0) tma_box(dst + oI, mI, bxI, byI, c.y, bar);
+                }
+                ++issued;
+                if (++r == NR) { r = 0; ++u; }
             }
-        }
-
-        // walking pointers into this kind's tables and this thread's partial sums
-        const float4* cp = reinterpret_cast<const float4*>(smem + prm.smem_coef_off[K]);
-        const int2* fp = reinterpret_cast<const int2*>(smem + prm.smem_fin_off[K]);
-        f2* const pp = s_part + tid;            // entry (q, j) at pp[(q * PP + j) * CONSUMERS]
-        const int uoff = slot_off(2 + K) / 4 + row * TX + 2 * lane;    // old value of pair 0 inside a step
-        // consumer step s is stage s (ring slot ring_r, phase ring_ph): its
-        // barrier is awaited before the step and released after it
-        auto stage_ptr = [&]() -> const float* {
-            if (alive) alive = wait_bounded(&full[ring_r], ring_ph, abort_flag, prm.err);
-            return reinterpret_cast<const float*>(ring + ring_r * STAGE_BYTES);
         };
-        auto stage_done = [&]() {
+        if (h == 1 && tl > 0 && prm.nclasses == 2) {
+            // the decay pairs (and the source) of this tile (not the first: there
+            // the consumers load them at once) into L2 while the consumers finish
+            // the previous tiles; lane = (kind, class, plane a / b, half row of 32)
+            issue(min(1, nst));
+            const int kind = lane >> 4, c = (lane >> 3) & 1, ab = (lane >> 2) & 1, hx = lane & 1;
+            const OutGrid& Gk = prm.out[kind];
+            const int x = x0 + 32 * hx;
+            if (x < Gk.nx) {
+                const long plane = (long)Gk.cp * Gk.ny;
+                // lanes with bit 1 clear: decay pairs; lanes 2 + 16 kind (+1): the kind's source
+                const float* base = ((lane >> 1) & 1) == 0
+                    ? (Gk.coef != nullptr ? Gk.coef + ((long)c * 4 + 2 * prm.which + ab) * plane + x : nullptr)
+                    : ((lane & 12) == 0 && prm.pf_src[kind] != nullptr ? prm.pf_src[kind] + x : nullptr);
+                if (base != nullptr)
+                    for (int y = y0; y < y0 + S::TY && y < Gk.ny; ++y)
+                        asm volatile("prefetch.global.L2 [%0];" ::"l"(base + (long)y * Gk.cp));
+            }
             __syncwarp();
-            if (lane == 0) mbar_arrive(&empty[ring_r]);
-            ++s;
-            if (++ring_r == NR) { ring_r = 0; ring_ph ^= 1u; }
-        };
-        // decay pairs (a, b) of the outputs of order L
-        f2 aL[PP], bL[PP];
-        auto set_order = [&](int L) {
-    #pragma unroll
-            for (int j = 0; j < PP; ++j) {
-                if (prm.nclasses == 2) {
-                    aL[j] = L == 0 ? ca2[j][0] : ca2[j][1];
-                    bL[j] = L == 0 ? cb2[j][0] : cb2[j][1];
-                } else {
-                    const float* cf = G.coef + (long)L * 4 * plane + cidxA[j];
-                    const float a0 = inA[j] ? __ldg(cf + 2 * prm.which * plane) : 0.f;
-                    const float b0 = inA[j] ? __ldg(cf + (2 * prm.which + 1) * plane) : 0.f;
-                    const float a1 = inB[j] ? __ldg(cf + 2 * prm.which * plane + 1) : 0.f;
-                    const float b1 = inB[j] ? __ldg(cf + (2 * prm.which + 1) * plane + 1) : 0.f;
-                    aL[j] = f2_make(a0, a1);
-                    bL[j] = f2_make(b0, b1);
-                }
-            }
-        };
-        // finalise this warp's output of the current finalising step (slot 2 + K)
-        auto finalize = [&](const float* t, const f2 (&W)[PP]) {
-            const int2 f = *fp;
-            fp += 1;
-    #pragma unroll
-            for (int j = 0; j < PP; ++j) {
-                const f2 u = lds2(t + uoff + out_off(j));
-                f2 w = W[j];
-                if (f.y >= 0) {
-                    const float* qs = prm.srcs[f.y];
-                    const float q0 = inA[j] ? __ldg(qs + cidxA[j]) : 0.f;
-                    const float q1 = inB[j] ? __ldg(qs + cidxA[j] + 1) : 0.f;
-                    w = f2_add(w, f2_make(q0, q1));
-                }
-                const f2 v = f2_fma(aL[j], u, f2_mul(bL[j], w));
-                if (f.x < 0 || !alive) continue;
-                float* dst = pptr[j] + 32 * (long)f.x;            // 64-bit: states beyond 2^31 values
-                // the pair with one 8-byte store; only a ragged right edge
-                // stores A alone
-                if (pair[j]) {
-                    *reinterpret_cast<f2*>(dst) = v;
-                } else if (inA[j]) {
-                    float v0, v1;
-                    f2_split(v, v0, v1);
-                    *dst = v0;
-                }
-            }
-        };
-        // accumulate a q step into the four targets of kind K in reach: d_x of
-        // the input of kind K (slot K), d_y of the other input (slot 1 - K);
-        // a missing I input has zero coefficients and its differences masked
-        auto accumulate = [&](const float* t, bool inI, f2 (&Pc)[PP], f2 (&Pn)[PP], f2 (&Nc)[PP], f2 (&Nn)[PP]) {
-            // each coefficient as an f32x2 pair (the same value for both points)
-            const float4 cxv = cp[0], cyv = cp[1];
-            cp += 2;
-            const f2 xPm = f2_make(cxv.x, cxv.x), xP0 = f2_make(cxv.y, cxv.y);
-            const f2 xN0 = f2_make(cxv.z, cxv.z), xNp = f2_make(cxv.w, cxv.w);
-            const f2 yPm = f2_make(cyv.x, cyv.x), yP0 = f2_make(cyv.y, cyv.y);
-            const f2 yN0 = f2_make(cyv.z, cyv.z), yNp = f2_make(cyv.w, cyv.w);
-    #pragma unroll
-            for (int j = 0; j < PP; ++j) {
-                f2 dx = diff_x(t + rx + in_off(j), cx, ev);
-                f2 dy = f2_sub(lds2(t + uy + in_off(j)), lds2(t + uy + in_off(j) - BX));
-                if (!inI) {
-                    if (K == 1) dx = zero2(); else dy = zero2();
-                }
-                Pc[j] = f2_fma(xPm, dx, Pc[j]);
-                Pn[j] = f2_fma(xP0, dx, Pn[j]);
-                Nc[j] = f2_fma(xN0, dx, Nc[j]);
-                Nn[j] = f2_fma(xNp, dx, Nn[j]);
-                Pc[j] = f2_fma(yPm, dy, Pc[j]);
-                Pn[j] = f2_fma(yP0, dy, Pn[j]);
-                Nc[j] = f2_fma(yN0, dy, Nc[j]);
-                Nn[j] = f2_fma(yNp, dy, Nn[j]);
-            }
-        };
-
-        const int N = prm.N;
-        const int first = 1 - prm.P;              // first input order: even l' for the odd pass
-        int last_in = first;
-        for (int lp = first; lp <= N && alive; lp += 2) {
-            last_in = lp;
-            const int nq = nq_of(lp);
-            const int nqp = nq_of(lp - 1);                    // previous-order targets
-            const int nqn = lp + 1 <= N ? nq_of(lp + 1) : 0;  // next-order targets
-            const int nqload = lp > first ? nqp : 0;          // previous-order partial sums exist once order lp - 2 passed
-            set_order(lp - 1);
-            f2 Pc[PP], Nc[PP], Pn[PP], Nn[PP];
-    #pragma unroll
-            for (int j = 0; j < PP; ++j) { Pc[j] = zero2(); Nc[j] = zero2(); }
-            // one q step: (Pc, Nc) carried in, (Pn, Nn) started here
-            auto qstep = [&](int q, f2 (&Pc_)[PP], f2 (&Nc_)[PP], f2 (&Pn_)[PP], f2 (&Nn_)[PP]) {
-    #pragma unroll
-                for (int j = 0; j < PP; ++j) {
-                    Pn_[j] = q < nqload ? pp[(q * PP + j) * CONSUMERS] : zero2();
-                    Nn_[j] = zero2();
-                }
-                const float* t = stage_ptr();
-                accumulate(t, has_imag(lp, q), Pc_, Pn_, Nc_, Nn_);
-                if (q >= 1 && q - 1 < nqp) finalize(t, Pc_);
-                stage_done();
-                if (q < nqn) {
-    #pragma unroll
-                    for (int j = 0; j < PP; ++j) pp[(q * PP + j) * CONSUMERS] = Nc_[j];
-                }
-            };
-            int q = 0;
-            for (; q + 1 < nq && alive; q += 2) {
-                qstep(q, Pc, Nc, Pn, Nn);
-                qstep(q + 1, Pn, Nn, Pc, Nc);
-            }
-            if (q < nq && alive) {
-                qstep(q, Pc, Nc, Pn, Nn);
-    #pragma unroll
-                for (int j = 0; j < PP; ++j) { Pc[j] = Pn[j]; Nc[j] = Nn[j]; }
-            }
-            if (alive && nq - 1 < nqp) {
-                // tail step: the last previous-order target
-                const float* t = stage_ptr();
-                finalize(t, Pc);
-                stage_done();
-            }
-            if (nq < nqn) {
-    #pragma unroll
-                for (int j = 0; j < PP; ++j) pp[(nq * PP + j) * CONSUMERS] = Nc[j];
-            }
         }
-        // outputs of the order above the last input order have no further inputs
-        const int L = last_in + 1;
-        if (L <= prm.top) {
-            set_order(L);
-            for (int q = 0; q < nq_of(L) && alive; ++q) {
-                f2 W[PP];
-    #pragma unroll
-                for (int j = 0; j < PP; ++j) W[j] = pp[(q * PP + j) * CONSUMERS];
-                const float* t = stage_ptr();
-                finalize(t, W);
-                stage_done();
-            }
-        }
-        // every tile consumes exactly the stages the producers issue for it
-        if (alive && s != (tl + 1) * prm.nstages) {
-            alive = false;
-            atomicExch(prm.err, 1);
+        issue(nst);
+    }
+    if (!ok && lane == 0) {
+        // aborted: wait (bounded) for the copies still in flight
+        for (int G = issued - 1; G >= 0 && G > issued - 1 - NR; --G) {
+            const unsigned long long tw = global_ns();
+            while (!mbar_try_wait(&full[G % NR], (G / NR) & 1))
+                if (global_ns() - tw > WAIT_NS) break;
         }
     }
 }
@@ -625,8 +830,10 @@ __device__ __forceinline__ void tiled_tiles(const Params& prm, const CUtensorMap
 // ... (raster order).  The CTAs then work on one contiguous band of tiles
 // at any time, so the halo rows that vertically adjacent tiles share come
 // from DRAM once, and each CTA's pipeline runs on across its tiles.
-__global__ void __launch_bounds__(THREADS, MINB) k_tiled_pass(const __grid_constant__ Params prm, int ntiles) {
-    tiled_tiles(prm, prm.maps, blockIdx.x, gridDim.x, ntiles, true);
+template <class S>
+__global__ void __launch_bounds__(S::THREADS, S::MINB) k_tiled_pass(const __grid_constant__ Params prm,
+                                                                                    int ntiles) {
+    tiled_tiles<S>(prm, prm.maps, blockIdx.x, gridDim.x, ntiles, true);
 }
 
 // Batched pass: CTA b runs items[off[b]] .. items[off[b + 1] - 1], each a
@@ -635,9 +842,11 @@ __global__ void __launch_bounds__(THREADS, MINB) k_tiled_pass(const __grid_const
 // parameters for parity P and coefficient set `which` are
 // prms[(2 i + P) * 2 + which] in global memory; the CTA copies them to
 // shared memory and hands TMA the tensor maps of the global copy.
-__global__ void __launch_bounds__(THREADS, MINB) k_tiled_batch(const Params* __restrict__ prms,
-                                                            const int4* __restrict__ items,
-                                                            const int* __restrict__ off, int P, int which) {
+template <class S>
+__global__ void __launch_bounds__(S::THREADS, S::MINB) k_tiled_batch(const Params* __restrict__ prms,
+                                                                                     const int4* __restrict__ items,
+                                                                                     const int* __restrict__ off,
+                                                                                     int P, int which) {
     __shared__ Params s_prm;
     const int begin = off[blockIdx.x], end = off[blockIdx.x + 1];
     for (int it = begin; it < end; ++it) {
@@ -650,9 +859,9 @@ __global__ void __launch_bounds__(THREADS, MINB) k_tiled_batch(const Params* __r
             for (int i = threadIdx.x; i < (int)(sizeof(Params) / 16); i += blockDim.x) dst[i] = src[i];
         }
         __syncthreads();
-        tiled_tiles(s_prm, g->maps, item.y, item.w, item.y + (item.z - 1) * item.w + 1, it == begin);
+        tiled_tiles<S>(s_prm, g->maps, item.y, item.w, item.y + (item.z - 1) * item.w + 1, it == begin);
     }
 }
 
-}  // namespace STARMAP_TILED_NS
+}  // namespace tiled
 }  // namespace starmap

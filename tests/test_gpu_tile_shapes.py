@@ -1,0 +1,82 @@
+"""The tile shapes of the FP32 kernel give the same values bit for bit: each
+point sees the same arithmetic in the same order whatever the tile height, the
+rows per warp and the CTAs per SM (the 5-row tiles are held to the oracle in
+test_gpu_tiled.py and test_gpu_edge.py)."""
+import numpy as np
+import pytest
+
+from paper_1211_2205_gb300 import capi
+from test_gpu_parity import _random_problem
+
+pytestmark = pytest.mark.gpu
+
+BCS = [("periodic", "periodic"), ("extrapolation", "extrapolation"), ("periodic", "extrapolation"),
+       ("extrapolation", "periodic")]
+
+
+def _state(p, kernel):
+    s = capi.Stepper.from_problem(p, kernel=kernel, schedule="merged")
+    s.step(p.nsteps)
+    return s.get_state()
+
+
+@pytest.mark.parametrize("bc", BCS)
+@pytest.mark.parametrize("N", [1, 2, 5, 15])
+def test_five_row_bands(N, bc):
+    """641 x 163 cells: 187 tiles of 64 x 10 (more than a GPU has SMs, so the
+    five-row bands), one column in the last tile column, three rows in the
+    last tile row (the second band empty), an odd width; four steps carry the
+    boundary copies back in."""
+    p = _random_problem(N, (641, 163), bc, "fp32", 900 + N, 4)
+    assert _state(p, "tiled_tall") == _state(p, "tiled_short")
+
+
+@pytest.mark.parametrize("n", [(64, 10), (65, 11), (63, 9), (2, 30), (3, 5), (130, 47)])
+@pytest.mark.parametrize("bc", BCS)
+def test_two_row_bands(n, bc):
+    """Grids of at most a tile per SM (two-row bands) around the tile's edges."""
+    p = _random_problem(6, n, bc, "fp32", 950, 4)
+    assert _state(p, "tiled_tall") == _state(p, "tiled_short")
+
+
+@pytest.mark.parametrize("N", [16, 49, 50, 55])
+def test_orders_around_the_table_limits(N):
+    """16: two-row bands whatever the grid; 49 / 50: weights kept twice /
+    once; 55: the highest order of the 10-row tiles."""
+    p = _random_problem(N, (70, 23), ("periodic", "extrapolation"), "fp32", 970, 2)
+    assert _state(p, "tiled_tall") == _state(p, "tiled_short")
+
+
+@pytest.mark.parametrize("bc", BCS)
+def test_boundary_copies(bc):
+    """After a step every boundary copy, corners included, holds the value it
+    copies (periodic: -1 <- n - 1, n <- 0; extrapolation: -1 <- 0, n <- n - 1;
+    none on an extrapolation axis of nodes)."""
+    import torch
+    p = _random_problem(3, (75, 12), bc, "fp32", 980, 1)
+    s = capi.Stepper.from_problem(p, kernel="tiled_tall", schedule="merged")
+    s.step(1)
+    s.sync()
+
+    class View:
+        pass
+
+    for j in range(s.ncomp):
+        i = s.moment_info(j)
+        ptr, pitch, off = s.device_ptr(j)
+        v = View()
+        v.__cuda_array_interface__ = dict(shape=(i["ny"] + 2, i["nx"] + 2), strides=(pitch * 4, 4), typestr="<f4",
+                                          data=(ptr + 4 * (off - pitch - 1), False), version=3)
+        a = torch.as_tensor(v, device="cuda").cpu().numpy()
+        u = a[1:-1, 1:-1]
+        node = (i["grid"] & 1, i["grid"] >> 1)
+        copies = [bc[d] == "periodic" or not node[d] for d in range(2)]
+        pad = u
+        for d, axis in ((0, 1), (1, 0)):
+            if copies[d]:
+                width = [(0, 0), (0, 0)]
+                width[axis] = (1, 1)
+                pad = np.pad(pad, width, mode="wrap" if bc[d] == "periodic" else "edge")
+        lo = [0 if c else 1 for c in copies]
+        got = a[lo[1]:a.shape[0] - lo[1], lo[0]:a.shape[1] - lo[0]]
+        assert np.array_equal(got, pad), (j, i)
