@@ -58,7 +58,8 @@ METRIC = "moment-cell updates/s"
 PAPER_UPDATES_PER_S = 18.3e6 / 1.5
 PROFILE_TRAFFIC = os.path.join(ROOT, "profiles", "roofline_traffic.json")
 KERNEL_SOURCES = {
-    "gather": ["paper_1211_2205_gb300/csrc/kernels_gather.cu"],
+    "gather": ["paper_1211_2205_gb300/csrc/kernels_gather.cu", "paper_1211_2205_gb300/csrc/kernels_stream.cu",
+               "paper_1211_2205_gb300/csrc/stream.h", "paper_1211_2205_gb300/csrc/pdl.h"],
     "tiled": ["paper_1211_2205_gb300/csrc/tiled.cu", "paper_1211_2205_gb300/csrc/tiled_kernel.cuh",
               "paper_1211_2205_gb300/csrc/pdl.h"],
 }
@@ -621,8 +622,8 @@ def run_native(args):
 
     clocks = clk.summary()
     steps_to_final = math.ceil(problem.t_final / s.dt - 1e-9) if problem.t_final else 0
-    # a tiled pass is one kernel, a gather pass one per output grid
-    launches = (2 * args.steps + 1) * (1 if s.kernel == "tiled" else 2)
+    # a pass is one kernel
+    launches = 2 * args.steps + 1
     if args.schedule == "fused":
         # O_1/2, the inner steps (fused launch + odd refresh each; an odd count
         # runs one as two passes), E and O_1/2

@@ -15,6 +15,7 @@
 #include "host_math.h"
 #include "internal.h"
 #include "mlp.h"
+#include "stream.h"
 #include "tiled.h"
 #include "../../include/starmap.h"
 
@@ -76,6 +77,7 @@ struct starmap_s {
     bool ghosts_dirty = true;
     int kernel_used = STARMAP_KERNEL_GATHER;
     TiledPlan* tiled = nullptr;
+    StreamTables* stream64 = nullptr;     // FP64 2D passes (null: the gather kernel)
     // learned closure (STARMAP_CLOSURE_MLP8)
     int closure = STARMAP_CLOSURE_NONE;
     int nsys = 0;                          // order of the assembled system
@@ -237,6 +239,12 @@ int build_tables(starmap_t* h) {
         int rc = tiled_update(h->tiled, h->sys, h->comp_class, h->src_slot, h->src_dev, h->frozen, h->dx, h->dy);
         if (rc) return fail(h, rc, tiled_error(h->tiled));
     }
+    if (!h->fp32 && h->cfg.system == STARMAP_PN2D) {
+        stream_destroy(h->stream64);
+        h->stream64 = nullptr;
+        if (stream_build(h->sys, h->comp_class, h->src_slot, h->frozen, h->dx, h->dy, &h->stream64))
+            return fail(h, STARMAP_E_CUDA, "cudaMalloc tables");
+    }
     ++h->version;
     return STARMAP_OK;
 }
@@ -325,22 +333,37 @@ int run_pass(starmap_t* h, bool odd, int which) {
         if (rc) return fail(h, rc, tiled_error(h->tiled));
         return STARMAP_OK;
     }
-    const int gl[2] = {odd ? 1 : 0, odd ? 2 : 3};
-    for (int q = 0; q < 2; ++q) {
-        GatherArgs<T> a;
-        for (int g = 0; g < 4; ++g) a.g[g] = grid_dev<T>(h, g);
+    if (h->stream64) {
+        StreamArgs a;
+        for (int g = 0; g < 4; ++g) a.g[g] = grid_dev<double>(h, g);
         a.pitch = h->pitch;
         a.p[0] = h->p[0];
         a.p[1] = h->p[1];
-        a.out_grid = gl[q];
-        a.begin = h->tbeg[gl[q]];
-        a.end = h->tend[gl[q]];
+        a.P = odd ? 1 : 0;
         a.which = which;
-        a.outs = h->outs_dev;
-        a.coefs = (const GatherCoef<T>*)h->coefs_dev;
-        a.src = (T* const*)h->src_ptrs_dev;
-        if (launch_gather_pass<T>(a, h->stream)) return cuda_fail(h, cudaGetLastError(), "gather pass");
+        a.src = (double* const*)h->src_ptrs_dev;
+        if (stream_pass(h->stream64, a, h->stream)) return cuda_fail(h, cudaGetLastError(), "FP64 pass");
+        return STARMAP_OK;
     }
+    GatherArgs<T> a;
+    for (int q = 0; q < 2; ++q) {
+        const int g = q == 0 ? (odd ? 1 : 0) : (odd ? 2 : 3);
+        a.out[q] = grid_dev<T>(h, g);
+        a.xin[q] = grid_dev<T>(h, g ^ 1);
+        a.yin[q] = grid_dev<T>(h, g ^ 2);
+        a.grid[q] = g;
+        a.begin[q] = h->tbeg[g];
+        a.end[q] = h->tend[g];
+        a.slices[q] = 0;
+    }
+    a.pitch = h->pitch;
+    a.p[0] = h->p[0];
+    a.p[1] = h->p[1];
+    a.which = which;
+    a.outs = h->outs_dev;
+    a.coefs = (const GatherCoef<T>*)h->coefs_dev;
+    a.src = (T* const*)h->src_ptrs_dev;
+    if (launch_gather_pass<T>(a, h->stream)) return cuda_fail(h, cudaGetLastError(), "gather pass");
     return STARMAP_OK;
 }
 
@@ -547,6 +570,7 @@ void release(starmap_t* h) {
     for (int g = 0; g < 4; ++g) if (h->snap[g]) cudaFree(h->snap[g]);
     for (int g = 0; g < 4; ++g) if (h->alloc1[g]) cudaFree(h->alloc1[g]);
     if (h->tiled) tiled_destroy(h->tiled);
+    stream_destroy(h->stream64);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
 }
 

@@ -65,11 +65,12 @@ struct GatherCoef { T cx[MAXC], cy[MAXC]; };
 
 template <class T>
 struct GatherArgs {
-    GridDev<T> g[4];
+    GridDev<T> out[2], xin[2], yin[2];   // the pass's output grids, and their partners staggered in x / y
+    int grid[2];                  // grid numbers of the outputs
+    int begin[2], end[2];         // ranges of output components in outs[]
+    int slices[2];                // of blockIdx.z (set by the launcher)
     long pitch;
     int p[2];                     // periodicity flags p_x, p_y
-    int out_grid;                 // grid updated by this launch
-    int begin, end;               // range of output components in outs[]
     int which;                    // 0: half-step coefficients, 1: full step
     const GatherOut* outs;
     const GatherCoef<T>* coefs;
@@ -103,7 +104,7 @@ struct ReduceArgs {
 };
 
 // launchers (kernels_gather.cu)
-template <class T> int launch_gather_pass(const GatherArgs<T>& a, void* stream);
+template <class T> int launch_gather_pass(GatherArgs<T> a, void* stream);
 template <class T> int launch_fill_ghosts(const GhostArgs<T>& a, void* stream);
 // overlap: programmatic dependent launch (after a short tiled pass)
 template <class T> int launch_fill_ghosts_pass(const GhostPassArgs<T>& a, void* stream, bool overlap);

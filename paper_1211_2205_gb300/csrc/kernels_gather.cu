@@ -129,47 +129,83 @@ __device__ __forceinline__ void ghost_item(T* comp, long pitch, int nx, int ny, 
     else if (i == 3) at(nx, ny) = at(xr, yhi);
 }
 
+// w + sum_k c[k] (p[k] - m[k]) over the first n of up to four terms, in
+// order, as straight lines: an FP64 operation predicated off takes its 64
+// clocks of the unit all the same.
 template <class T>
-__global__ void k_gather_pass(const GatherArgs<T> A) {
-    const int g = A.out_grid;
-    const GridDev<T>& G = A.g[g];
-    const int ix = blockIdx.x * blockDim.x + threadIdx.x;
-    const int iy = blockIdx.y;
-    if (ix >= G.nx || iy >= G.ny) return;
-    const bool xnode = (g & 1) != 0, ynode = (g & 2) != 0;
-    const int xg = g ^ 1, yg = g ^ 2;                  // partner grids
+__device__ __forceinline__ T add_terms(T w, int n, const T (&c)[MAXC], const T (&p)[MAXC], const T (&m)[MAXC]) {
+    static_assert(MAXC == 4, "up to four couplings per direction");
+    switch (n) {
+        case 4:
+            return w + c[0] * (p[0] - m[0]) + c[1] * (p[1] - m[1]) + c[2] * (p[2] - m[2]) + c[3] * (p[3] - m[3]);
+        case 3: return w + c[0] * (p[0] - m[0]) + c[1] * (p[1] - m[1]) + c[2] * (p[2] - m[2]);
+        case 2: return w + c[0] * (p[0] - m[0]) + c[1] * (p[1] - m[1]);
+        case 1: return w + c[0] * (p[0] - m[0]);
+        default: return w;
+    }
+}
+
+// Both output grids of a pass in one launch: blockIdx.z = slice, the first
+// A.slices[0] of them on output grid 0, the others on grid 1; output t of a
+// grid goes to slice (t - begin) mod slices.  On small grids, where a thread
+// has one output, the launch, a table load and a chain of loads and FP64
+// operations (64 clocks each, one at a time per warp) are the pass: the
+// tables and decay coefficients, host-written, are loaded before the
+// previous pass is waited for (pdl.h).
+template <class T>
+__global__ void __launch_bounds__(128) k_gather_pass(const __grid_constant__ GatherArgs<T> A) {
+    pdl_trigger();
+    const int K = (int)blockIdx.z < A.slices[0] ? 0 : 1;
+    const int slice = (int)blockIdx.z - (K ? A.slices[0] : 0);
+    const GridDev<T>& G = A.out[K];
+    const int nx = G.nx, ny = G.ny;
+    // points in rows one after the other: no lanes idle at a row's end (an FP64 operation costs a warp of
+    // four lanes what it costs a whole one)
+    const unsigned long long point = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const bool inside = point < (unsigned long long)nx * ny;
+    const int iy = point >> 32 ? (int)(point / nx) : (int)((unsigned)point / (unsigned)nx);
+    const int ix = (int)(point - (unsigned long long)iy * nx);
+    const bool xnode = (A.grid[K] & 1) != 0, ynode = (A.grid[K] & 2) != 0;
     const long pitch = A.pitch;
-    // right / upper neighbour index in the partner grid (eq. central_differences)
-    const int xr = ix + (xnode ? A.p[0] : 1 - A.p[0]);
-    const int yu = iy + (ynode ? A.p[1] : 1 - A.p[1]);
-    const long o_r = (long)(iy + 1) * pitch + xr;
-    const long o_u = (long)(yu + 1) * pitch + ix;
-    const long o_self = (long)(iy + 1) * pitch + ix;
-    const long cidx = (long)iy * G.cp + ix;
-    const long plane = (long)G.cp * G.ny;
-    const T* Xb = A.g[xg].base;
-    const T* Yb = A.g[yg].base;
-    const long cxs = A.g[xg].cstride, cys = A.g[yg].cstride;
-    for (int t = A.begin + (int)blockIdx.z; t < A.end; t += (int)gridDim.z) {
+    // right / upper neighbour in the partner grid (eq. central_differences)
+    const T* Xb = A.xin[K].base + (long)(iy + 1) * pitch + ix + (xnode ? A.p[0] : 1 - A.p[0]);
+    const T* Yb = A.yin[K].base + (long)(iy + 1 + (ynode ? A.p[1] : 1 - A.p[1])) * pitch + ix;
+    const long cxs = A.xin[K].cstride, cys = A.yin[K].cstride;
+    T* self = G.base + (long)(iy + 1) * pitch + ix;
+    const long cidx = inside ? (long)iy * G.cp + ix : 0;
+    const long plane = (long)G.cp * ny;
+    bool waited = false;
+    for (int t = A.begin[K] + slice; t < A.end[K]; t += A.slices[K]) {
         const GatherOut o = A.outs[t];
         const GatherCoef<T> c = A.coefs[t];
-        T w = T(0);
-        for (int k = 0; k < o.nxt; ++k) {
-            const T* b = Xb + (long)o.xin[k] * cxs;
-            w += c.cx[k] * (b[o_r] - b[o_r - 1]);
+        const T* cf = G.coef + ((long)o.cls * 4 + 2 * A.which) * plane + cidx;
+        const T a = cf[0];
+        const T bb = cf[plane];
+        const T q = o.src >= 0 ? A.src[o.src][cidx] : T(0);
+        if (!waited) {
+            pdl_wait();
+            waited = true;
         }
-        for (int k = 0; k < o.nyt; ++k) {
-            const T* b = Yb + (long)o.yin[k] * cys;
-            w += c.cy[k] * (b[o_u] - b[o_u - pitch]);
+        if (!inside) continue;
+        T r[MAXC], l[MAXC], u[MAXC], d[MAXC];
+#pragma unroll
+        for (int k = 0; k < MAXC; ++k) {
+            const T* x = Xb + (long)o.xin[k] * cxs;
+            const T* y = Yb + (long)o.yin[k] * cys;
+            r[k] = k < o.nxt ? x[0] : T(0);
+            l[k] = k < o.nxt ? x[-1] : T(0);
+            u[k] = k < o.nyt ? y[0] : T(0);
+            d[k] = k < o.nyt ? y[-pitch] : T(0);
         }
-        if (o.src >= 0) w += A.src[o.src][cidx];
-        const T* cf = G.coef + (long)o.cls * 4 * plane + cidx;
-        const T a = cf[(2 * A.which) * plane];
-        const T bb = cf[(2 * A.which + 1) * plane];
         T* comp = G.base + (long)o.local * G.cstride;
-        const T v = a * comp[o_self] + bb * w;
-        store_point(comp, pitch, ix, iy, G.nx, G.ny, xnode, ynode, A.p[0], A.p[1], v);
+        const T old = self[(long)o.local * G.cstride];
+        T w = add_terms<T>(T(0), o.nxt, c.cx, r, l);
+        w = add_terms<T>(w, o.nyt, c.cy, u, d);
+        if (o.src >= 0) w += q;
+        const T v = a * old + bb * w;
+        store_point(comp, pitch, ix, iy, nx, ny, xnode, ynode, A.p[0], A.p[1], v);
     }
+    if (!waited) pdl_wait();
 }
 
 // Refresh the boundary copies of components [kbegin, kend) of one grid.
@@ -293,21 +329,29 @@ static int sm_count_gather() {
 }
 
 template <class T>
-int launch_gather_pass(const GatherArgs<T>& a, void* stream) {
-    const GridDev<T>& G = a.g[a.out_grid];
-    if (a.end <= a.begin || G.nx == 0 || G.ny == 0) return 0;
-    dim3 block(128);
-    // one thread per point walks the grid's outputs; on a small grid the
-    // outputs are dealt over blockIdx.z as well (output t to slice (t - begin)
-    // mod z), so that about two waves of threads fill the GPU
-    const long threads = (long)((G.nx + 127) / 128) * 128 * G.ny;
+int launch_gather_pass(GatherArgs<T> a, void* stream) {
+    long points = 0;
+    int outs = 0;
+    for (int K = 0; K < 2; ++K) {
+        if (a.end[K] <= a.begin[K]) continue;
+        points = std::max(points, (long)a.out[K].nx * a.out[K].ny);
+        outs += a.end[K] - a.begin[K];
+    }
+    if (outs == 0 || points == 0) return 0;
+    // one thread per point walks a slice of a grid's outputs; on a small grid
+    // the outputs are dealt over more slices, so that about two waves of
+    // threads fill the GPU
+    const int width = 128;
+    const long threads = (points + width - 1) / width * width;
     const long want = 2L * 2048 * sm_count_gather();
-    long z = threads >= want ? 1 : (want + threads - 1) / threads;
-    if (z > a.end - a.begin) z = a.end - a.begin;
-    if (z > 64) z = 64;
-    dim3 grid((G.nx + 127) / 128, G.ny, (unsigned)z);
-    k_gather_pass<T><<<grid, block, 0, (cudaStream_t)stream>>>(a);
-    return status_of(cudaGetLastError());
+    for (int K = 0; K < 2; ++K) {
+        const int n = a.end[K] - a.begin[K];
+        const long z = threads >= want ? 1 : (want * std::max(n, 0) / outs + threads - 1) / threads;
+        a.slices[K] = n <= 0 ? 0 : (int)std::min<long>(std::min<long>(std::max<long>(z, 1), n), 64);
+    }
+    const dim3 grid((unsigned)(threads / width), 1, a.slices[0] + a.slices[1]);
+    const cudaError_t e = launch_pdl(k_gather_pass<T>, grid, dim3(width), 0, (cudaStream_t)stream, threads < want, a);
+    return status_of(e != cudaSuccess ? e : cudaGetLastError());
 }
 
 template <class T>
@@ -348,8 +392,8 @@ int launch_axpby(T* out, const T* x, const T* y, double alpha, double beta, size
     return status_of(cudaGetLastError());
 }
 
-template int launch_gather_pass<float>(const GatherArgs<float>&, void*);
-template int launch_gather_pass<double>(const GatherArgs<double>&, void*);
+template int launch_gather_pass<float>(GatherArgs<float>, void*);
+template int launch_gather_pass<double>(GatherArgs<double>, void*);
 template int launch_fill_ghosts<float>(const GhostArgs<float>&, void*);
 template int launch_fill_ghosts<double>(const GhostArgs<double>&, void*);
 template int launch_fill_ghosts_pass<float>(const GhostPassArgs<float>&, void*, bool);
