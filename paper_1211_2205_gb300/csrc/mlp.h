@@ -36,6 +36,13 @@ constexpr int OFF_W3 = OFF_B2 + HID;
 constexpr int OFF_B3 = OFF_W3 + NOUT * HID;
 constexpr int NPARAM = OFF_B3 + NOUT;        // 22665
 
+// Partial gradients of a tile: the parameter vector's order, but W1 and W2
+// transposed ([i][o]), so that the lanes of a warp, which own one output o
+// each, write runs of 128 bytes; the loss behind it.
+constexpr int PART_PITCH = (NPARAM + 1 + 31) / 32 * 32;
+constexpr int slot_w1(int o, int i) { return OFF_W1 + i * HID + o; }
+constexpr int slot_w2(int o, int i) { return OFF_W2 + i * HID + o; }
+
 // BF16 weights in the padded layout the kernels stage into shared memory.
 struct alignas(16) Packed {
     __nv_bfloat16 W1[HID * LDX];
@@ -61,14 +68,19 @@ int pack(const float* params, Packed* P, void* stream);
 int forward(const float* X, long M, const Packed* P, float* Y, void* stream);
 // Per-CTA partial gradients (and losses) of the mean squared error over the
 // B samples idx[0..B) (idx NULL: samples 0..B); part holds
-// blocks(B) x (NPARAM + 1) floats, reduced into grad[NPARAM], loss[1].
+// grad_blocks(B) x PART_PITCH floats.
 // engine: ENGINE_MMA_SYNC (mma.sync tiles) or ENGINE_TCGEN05 (tcgen05 tiles;
 // err: device flag raised by a bounded wait).
-int loss_grad(const float* X, const float* T, const int* idx, long B, const Packed* P, float* part, float* grad,
-              float* loss, int engine, int* err, void* stream);
+int loss_grad_tiles(const float* X, const float* T, const int* idx, long B, const Packed* P, float* part, int engine,
+                    int* err, void* stream);
 long grad_blocks(long B);
-int adam(float* p, const float* g, float* m, float* v, int n, float lr, float b1, float b2, float eps, long step,
-         void* stream);
+// Their sum over the tiles, into grad[NPARAM] and (not NULL) loss[1].
+int reduce_grad(const float* part, long tiles, float* grad, float* loss, void* stream);
+// The same sum as the gradient of Adam step number `step` on the parameters
+// p, which it writes to P too; m and v in the order of the partial gradients.
+// Follows loss_grad_tiles on the stream.
+int reduce_adam(const float* part, long tiles, float* loss, float* p, float* m, float* v, Packed* P, float lr, float b1,
+                float b2, float eps, long step, void* stream);
 // Xn = X with N(0, sigma^2) noise on the first `cols` of the NIN inputs of
 // each of the M rows (counter-based: the same seed gives the same noise).
 int perturb(const float* X, float* Xn, long M, int cols, float sigma, unsigned long long seed, void* stream);

@@ -20,9 +20,8 @@ struct starmap_mlp_s {
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     float* params = nullptr;       // FP32 master parameters
-    float* m = nullptr;            // Adam first moment
-    float* v = nullptr;            // Adam second moment
-    float* grad = nullptr;         // gradient of the last train step
+    float* m = nullptr;            // Adam first moment, in the order of the partial gradients
+    float* v = nullptr;            // Adam second moment, likewise
     mlp::Packed* packed = nullptr; // BF16 copy used by the kernels
     float* part = nullptr;         // per-tile partial gradients
     long part_tiles = 0;
@@ -51,7 +50,6 @@ void mrelease(starmap_mlp_t* n) {
     cudaFree(n->params);
     cudaFree(n->m);
     cudaFree(n->v);
-    cudaFree(n->grad);
     cudaFree(n->packed);
     cudaFree(n->part);
     cudaFree(n->flag);
@@ -84,8 +82,16 @@ int ensure_part(starmap_mlp_t* net, long tiles) {
         net->part = nullptr;
         net->part_tiles = 0;
     }
-    MCK(dev_alloc(&net->part, (size_t)tiles * (mlp::NPARAM + 1) * sizeof(float)), "cudaMalloc gradient scratch");
+    MCK(dev_alloc(&net->part, (size_t)tiles * mlp::PART_PITCH * sizeof(float)), "cudaMalloc gradient scratch");
     net->part_tiles = tiles;
+    return STARMAP_OK;
+}
+
+// partial loss and gradients of the tiles of B samples
+int tile_grads(starmap_mlp_t* net, const float* X, const float* T, const int32_t* idx, size_t B) {
+    if (int rc = ensure_part(net, mlp::grad_blocks((long)B))) return rc;
+    if (mlp::loss_grad_tiles(X, T, idx, (long)B, net->packed, net->part, net->engine, net->flag, net->stream))
+        MCK(cudaGetLastError(), "loss_grad");
     return STARMAP_OK;
 }
 
@@ -115,7 +121,7 @@ int starmap_mlp_create(const float* params, size_t count, void* cuda_stream, sta
         net->own_stream = true;
     }
     const size_t pb = (size_t)mlp::NPARAM * sizeof(float);
-    float** bufs[4] = {&net->params, &net->m, &net->v, &net->grad};
+    float** bufs[3] = {&net->params, &net->m, &net->v};
     for (float** b : bufs) {
         e = dev_alloc(b, pb);
         if (e != cudaSuccess) return bail(mfail(net, STARMAP_E_NOMEM, "cudaMalloc parameters"));
@@ -169,8 +175,8 @@ int starmap_mlp_loss_grad(starmap_mlp_t* net, const float* X, const float* T, co
                           float* grad, float* loss) {
     if (!net) return STARMAP_E_ARG;
     if (B == 0 || !X || !T || !grad) return mfail(net, STARMAP_E_ARG, "loss_grad needs B > 0 and X, T, grad");
-    if (int rc = ensure_part(net, mlp::grad_blocks((long)B))) return rc;
-    if (mlp::loss_grad(X, T, idx, (long)B, net->packed, net->part, grad, loss, net->engine, net->flag, net->stream))
+    if (int rc = tile_grads(net, X, T, idx, B)) return rc;
+    if (mlp::reduce_grad(net->part, mlp::grad_blocks((long)B), grad, loss, net->stream))
         MCK(cudaGetLastError(), "loss_grad");
     return STARMAP_OK;
 }
@@ -179,12 +185,12 @@ int starmap_mlp_train_step(starmap_mlp_t* net, const float* X, const float* T, c
                            float* loss) {
     if (!net) return STARMAP_E_ARG;
     if (!(lr > 0.f) || !std::isfinite(lr)) return mfail(net, STARMAP_E_ARG, "learning rate must be positive");
-    if (int rc = starmap_mlp_loss_grad(net, X, T, idx, B, net->grad, loss)) return rc;
+    if (B == 0 || !X || !T) return mfail(net, STARMAP_E_ARG, "loss_grad needs B > 0 and X, T, grad");
+    if (int rc = tile_grads(net, X, T, idx, B)) return rc;
     net->steps += 1;
-    if (mlp::adam(net->params, net->grad, net->m, net->v, mlp::NPARAM, lr, ADAM_B1, ADAM_B2, ADAM_EPS, net->steps,
-                  net->stream))
+    if (mlp::reduce_adam(net->part, mlp::grad_blocks((long)B), loss, net->params, net->m, net->v, net->packed, lr,
+                         ADAM_B1, ADAM_B2, ADAM_EPS, net->steps, net->stream))
         MCK(cudaGetLastError(), "adam");
-    if (mlp::pack(net->params, net->packed, net->stream)) MCK(cudaGetLastError(), "pack");
     return STARMAP_OK;
 }
 

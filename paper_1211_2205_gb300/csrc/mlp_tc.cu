@@ -718,38 +718,42 @@ __global__ void k_tc_wait_selftest(int* err, int* result) {
 // operand (transpose bit of the instruction descriptor).  The bias gradients
 // b1 and b2 come out of the same MMAs: X and H1 carry a column of ones, so
 // dW1 and dW2 gain a column sum_s dZ[s][o].
-constexpr int TR_THREADS = 256;          // two warps per TMEM lane quarter, each one half of the columns
+constexpr int TR_THREADS = 512;          // G groups of them, a tile each
 constexpr int H1K = HID + 16;            // H1 columns: the hidden values, a ones column, zeros
 constexpr int H1_BYTES = (H1K / 8) * (TM / 8) * 128;        // 36864
 constexpr int DY_BYTES = (OUTP / 8) * (TM / 8) * 128;       // 4096
 constexpr int ONES_X = NIN;              // X column holding 1: b1's gradient in dW1's column NIN
 constexpr int ONES_H = HID;              // H1 column holding 1: b2's gradient in dW2's column HID
-constexpr uint32_t TC_ACC = 0;           // TMEM: forward accumulators, then dH2, then dH1 (128 columns)
+// a group's TMEM columns
+constexpr uint32_t TC_ACC = 0;           // forward accumulators, then dH2, then dH1 (128 columns)
 constexpr uint32_t TC_DW3 = 128;         // dW3^T (16 columns)
-constexpr uint32_t TC_DW2 = 256;         // dW2 and b2's gradient (144 columns)
-constexpr uint32_t TC_DW1 = 400;         // dW1 and b1's gradient (48 columns)
-static_assert(TC_DW1 + KX_TC <= TMEM_COLS, "the training accumulators fit in TMEM");
-// Layout order matters for nothing but keeps every operand's MN-major
-// reading inside the CTA's allocation: the buffers read that way (W3, dY,
-// X, H1, H2) are followed by at least 32 KB of the others.
-struct TrSmem {
-    alignas(128) unsigned char w1[W1_BYTES];    // W1 [o][i], K = 48
-    alignas(128) unsigned char w2[W2_BYTES];    // W2 [o][i]
-    alignas(128) unsigned char w3[W3_BYTES];    // W3 [o (16)][i]
+constexpr uint32_t TC_DW2 = 128;         // then dW2 (128 columns)
+constexpr uint32_t TC_DW1 = 0;           // dW1 and b1's gradient (48 columns), over dH1
+constexpr uint32_t TC_DB2 = 48;          // b2's gradient in the first of 16 columns
+constexpr uint32_t TR_COLS = 256;
+// Every operand's reading, K-major or MN-major, spans its buffer exactly.
+struct TrGroup {
     alignas(128) unsigned char dy[DY_BYTES];    // dY [s][o (16)]
     alignas(128) unsigned char x[XC_BYTES];     // X [s][48]
     alignas(128) unsigned char h1[H1_BYTES];    // H1 [s][144], later dZ1 in its first 128 columns
     alignas(128) unsigned char h2[H_BYTES];     // H2 [s][128], later dZ2
+    float wloss[GWARPS];
+    float wb3[GWARPS][OUTP];
+    alignas(8) uint64_t bar;
+    int stop;
+};
+template <int G>
+struct TrSmem {
+    alignas(128) unsigned char w1[W1_BYTES];    // W1 [o][i], K = 48
+    alignas(128) unsigned char w2[W2_BYTES];    // W2 [o][i]
+    alignas(128) unsigned char w3[W3_BYTES];    // W3 [o (16)][i]
+    TrGroup grp[G];
     alignas(16) float b1[HID];
     alignas(16) float b2[HID];
     alignas(16) float b3[OUTP];
-    float wloss[TR_THREADS / 32];
-    float wb3[GWARPS][OUTP];
-    alignas(8) uint64_t bar;
     uint32_t tmem;
-    int stop;
 };
-static_assert(sizeof(TrSmem) <= 227 * 1024, "training kernel shared memory");
+static_assert(sizeof(TrSmem<2>) <= 227 * 1024, "training kernel shared memory");
 
 // instruction descriptor with the operands' majorness: ta / tb = 1 reads A / B MN-major
 __host__ __device__ constexpr uint32_t idesc_t(int m, int n, int ta, int tb) {
@@ -771,38 +775,63 @@ __device__ __forceinline__ void mma_k(uint32_t d, uint64_t a, uint64_t as, uint6
     for (int kk = 0; kk < ksteps; ++kk) mma_f16(d, a + kk * as, b + kk * bs, id, kk > 0);
 }
 
-// Thread 0 commits the MMAs it issued and waits for them; every thread then
-// learns whether to stop.  Returns false if a wait expired.
-__device__ __forceinline__ bool tr_sync_mma(TrSmem& S, uint32_t& ph, int* err) {
-    if (threadIdx.x == 0) {
+template <int G>
+__device__ __forceinline__ void tr_sync(int g) {
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "n"(TR_THREADS / G) : "memory");
+}
+// The group's leader commits the MMAs it issued and waits for them; every
+// thread then learns whether to stop.  Returns false if a wait expired.
+template <int G>
+__device__ __forceinline__ bool tr_sync_mma(TrGroup& S, int g, bool leader, uint32_t& ph, int* err) {
+    if (leader) {
         mma_commit(&S.bar);
         if (!mbar_wait(&S.bar, ph & 1, err)) S.stop = 1;
     }
     ++ph;
-    __syncthreads();
+    tr_sync<G>(g);
     fence_after();
     return S.stop == 0;
 }
 // Before the next MMAs read what the threads wrote: generic -> async proxy,
 // TMEM reads ordered before the MMAs that overwrite the columns.
-__device__ __forceinline__ void tr_publish() {
+template <int G>
+__device__ __forceinline__ void tr_publish(int g) {
     fence_async_smem();
     fence_before();
-    __syncthreads();
+    tr_sync<G>(g);
     fence_after();
 }
 
-// dZ = dH * (1 - H^2) for the thread's row and 64 columns starting at c0:
-// dH from TMEM, H (BF16) read from and dZ written over the natural buffer
-__device__ __forceinline__ void tanh_backward(unsigned char* buf, uint32_t tacc, int row, int c0) {
+// H = tanh(Z + b) of the thread's row and its 32 G columns from c0, Z in TMEM
+template <int G>
+__device__ __forceinline__ void tanh_forward(unsigned char* buf, uint32_t tacc, const float* bias, int row, int first) {
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
+    for (int c0 = first; c0 < first + 32 * G; c0 += 32) {
         uint32_t v[32];
-        tmem_ld32(tacc + (uint32_t)(c0 + 32 * q), v);
+        tmem_ld32(tacc + (uint32_t)c0, v);
         tmem_wait_ld();
 #pragma unroll
         for (int cb = 0; cb < 32; cb += 8) {
-            uint4* at = reinterpret_cast<uint4*>(buf + canon(row, c0 + 32 * q + cb, TM));
+            uint32_t w[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                w[e] = bias_act2_tc(v[cb + 2 * e], v[cb + 2 * e + 1], bias[c0 + cb + 2 * e], bias[c0 + cb + 2 * e + 1]);
+            *reinterpret_cast<uint4*>(buf + canon(row, c0 + cb, TM)) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+    }
+}
+// dZ = dH * (1 - H^2) for the thread's row and its 32 G columns from c0: dH
+// from TMEM, H (BF16) read from and dZ written over the natural buffer
+template <int G>
+__device__ __forceinline__ void tanh_backward(unsigned char* buf, uint32_t tacc, int row, int first) {
+#pragma unroll
+    for (int c0 = first; c0 < first + 32 * G; c0 += 32) {
+        uint32_t v[32];
+        tmem_ld32(tacc + (uint32_t)c0, v);
+        tmem_wait_ld();
+#pragma unroll
+        for (int cb = 0; cb < 32; cb += 8) {
+            uint4* at = reinterpret_cast<uint4*>(buf + canon(row, c0 + cb, TM));
             const uint4 hv = *at;
             const uint32_t hw[4] = {hv.x, hv.y, hv.z, hv.w};
             uint32_t w[4];
@@ -818,28 +847,71 @@ __device__ __forceinline__ void tanh_backward(unsigned char* buf, uint32_t tacc,
     }
 }
 
+// Bound by latency: one tile is a chain of seven contractions with an
+// epilogue each, on one CTA per SM.  So the rows are read by runs of lanes
+// along them, the partial gradients leave by runs of 128 bytes while the next
+// contraction runs, and sixteen warps share each epilogue.  64 tiles (8192
+// samples, cold): 27 us with eight warps that read and wrote one row each
+// (32 sectors per instruction), 16 us so.  Beyond one tile per SM a CTA takes
+// two, each a group's, on one copy of the weights: 235 tiles 52 -> 23 us.
+template <int G>
 __global__ void __launch_bounds__(TR_THREADS, 1) k_loss_grad_tc(const float* __restrict__ X, const float* __restrict__ T,
                                                                 const int* __restrict__ idx, long B,
                                                                 const Packed* __restrict__ P, float* __restrict__ part,
                                                                 int* __restrict__ err) {
     extern __shared__ __align__(1024) unsigned char raw[];
-    TrSmem& S = *reinterpret_cast<TrSmem*>(raw);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int quarter = warp % GWARPS, half = warp / GWARPS;
+    TrSmem<G>& W = *reinterpret_cast<TrSmem<G>*>(raw);
+    constexpr int GT = TR_THREADS / G;                   // threads of a group
+    constexpr int COLS = HID / (GT / TM);                // a thread's columns in an epilogue
+    const int g = threadIdx.x / GT, t = threadIdx.x % GT;
+    TrGroup& S = W.grp[g];
+    const int lane = threadIdx.x & 31;
+    const int quarter = (t >> 5) % GWARPS, share = t / TM;
     const int row = 32 * quarter + lane;                 // TMEM lane: a sample, or an output / input index
-    const long row0 = (long)blockIdx.x * TM;
-    float* out = part + (long)blockIdx.x * (NPARAM + 1);
-    if (threadIdx.x == 0) {
+    const int c0 = COLS * share;
+    const long tile = (long)blockIdx.x * G + g;
+    const long row0 = tile * TM;
+    const bool leader = t == 0;
+    float* out = part + tile * PART_PITCH;
+    if (leader) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(&S.bar)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         S.stop = 0;
     }
-    if (warp == 0)
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&S.tmem)),
-                     "r"(TMEM_COLS) : "memory");
-    // weights (natural layouts; Packed's padding columns are zero)
+    if (threadIdx.x < 32)
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&W.tmem)),
+                     "r"(TR_COLS * G) : "memory");
+    // H1's ones column and zeros behind it
+    if (t < 2 * TM) {
+        const int side = t / TM;
+        const uint32_t one = pack_bf16_tc(1.f, 0.f);
+        *reinterpret_cast<uint4*>(S.h1 + canon(t % TM, HID + 8 * side, TM)) =
+            side == 0 ? make_uint4(one, 0u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
+    }
+    // every buffer of the caller's, the weights and the parts may be the
+    // previous kernels'; the next kernel starts no earlier than this, so what
+    // precedes this grid is complete for it
+    pdl_wait();
+    pdl_trigger();
+    // sample rows (gathered through idx), a ones column, zeros: a pair of columns per thread and turn
     {
-        const uint32_t w1 = su32(S.w1), w2 = su32(S.w2), w3 = su32(S.w3);
+        constexpr int PAIRS = KX_TC / 2, TURNS = TM * PAIRS / GT;
+        static_assert(TM * PAIRS % GT == 0, "whole turns");
+        float v[TURNS][2];
+#pragma unroll
+        for (int k = 0; k < TURNS; ++k) {
+            const int i = t + k * GT, col = 2 * (i % PAIRS);
+            const long m = row0 + i / PAIRS;
+            v[k][0] = col == ONES_X ? 1.f : 0.f;
+            v[k][1] = 0.f;
+            if (m < B && col < NIN) {
+                const float* xs = X + (idx ? (long)idx[m] : m) * NIN + col;
+                v[k][0] = xs[0];
+                v[k][1] = xs[1];
+            }
+        }
+        // weights (natural layouts; Packed's padding columns are zero)
+        const uint32_t w1 = su32(W.w1), w2 = su32(W.w2), w3 = su32(W.w3);
         for (int i = threadIdx.x; i < HID * (KX_TC / 8); i += TR_THREADS) {
             const int n = i / (KX_TC / 8), c = i % (KX_TC / 8);
             cp_async16_tc(w1 + canon(n, 8 * c, HID), P->W1 + n * LDX + 8 * c);
@@ -853,124 +925,92 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_loss_grad_tc(const float* __r
             cp_async16_tc(w3 + canon(n, 8 * c, OUTP), P->W3 + n * LDH + 8 * c);
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
-        for (int i = threadIdx.x; i < HID; i += TR_THREADS) { S.b1[i] = P->b1[i]; S.b2[i] = P->b2[i]; }
-        if (threadIdx.x < OUTP) S.b3[threadIdx.x] = P->b3[threadIdx.x];
-    }
-    // inputs: sample rows (gathered through idx), a ones column, zeros; H1's
-    // ones column and zeros behind it
-    {
-        const int r = threadIdx.x % TM, side = threadIdx.x / TM;        // half a row each
-        const long m = row0 + r;
-        const bool ok = m < B;
-        const float* xs = X + (ok ? (idx ? (long)idx[m] : m) : 0) * NIN;
+        if (threadIdx.x < HID) { W.b1[threadIdx.x] = P->b1[threadIdx.x]; W.b2[threadIdx.x] = P->b2[threadIdx.x]; }
+        if (threadIdx.x < OUTP) W.b3[threadIdx.x] = P->b3[threadIdx.x];
 #pragma unroll
-        for (int c = 3 * side; c < 3 * side + 3; ++c) {
-            uint32_t w[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                float v[2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int col = 8 * c + 2 * e + h;
-                    v[h] = col < NIN ? (ok ? xs[col] : 0.f) : col == ONES_X ? 1.f : 0.f;
-                }
-                w[e] = pack_bf16_tc(v[0], v[1]);
-            }
-            *reinterpret_cast<uint4*>(S.x + canon(r, 8 * c, TM)) = make_uint4(w[0], w[1], w[2], w[3]);
+        for (int k = 0; k < TURNS; ++k) {
+            const int i = t + k * GT;
+            *reinterpret_cast<uint32_t*>(S.x + canon(i / PAIRS, 2 * (i % PAIRS), TM)) = pack_bf16_tc(v[k][0], v[k][1]);
         }
-        const uint32_t one = pack_bf16_tc(1.f, 0.f);
-        *reinterpret_cast<uint4*>(S.h1 + canon(r, HID + 8 * side, TM)) =
-            side == 0 ? make_uint4(one, 0u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
     }
     // the targets of the thread's sample (rows of the output epilogue), loaded
     // now so that their latency hides behind the forward layers
     float tgt[NOUT];
     {
         const long m = row0 + row;
-        const bool valid = half == 0 && m < B;
+        const bool valid = share == 0 && m < B;
         const float* ts = T + (valid ? (idx ? (long)idx[m] : m) : 0) * NOUT;
 #pragma unroll
         for (int o = 0; o < NOUT; ++o) tgt[o] = valid ? ts[o] : 0.f;
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
+    fence_async_smem();
     fence_before();
-    tr_publish();
-    const uint32_t tm = S.tmem;
+    __syncthreads();
+    fence_after();
+    const uint32_t tm = W.tmem + TR_COLS * g;
     const uint32_t tl = tm + ((uint32_t)(32 * quarter) << 16);      // this warp's lane quarter, column 0
     uint32_t ph = 0;
-    bool ok = true;
+    bool ok = row0 < B;              // the last CTA may have a group without a tile
     // ---- forward: Z1 = X W1^T, H1 = tanh(Z1 + b1)
-    if (threadIdx.x == 0) mma_k(tm + TC_ACC, kdesc(su32(S.x), TM), kstep(TM), kdesc(su32(S.w1), HID), kstep(HID),
-                                idesc(TM, HID), KX_TC / 16);
-    ok = tr_sync_mma(S, ph, err);
     if (ok) {
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int c0 = 64 * half + 32 * q;
-            uint32_t v[32];
-            tmem_ld32(tl + TC_ACC + (uint32_t)c0, v);
-            tmem_wait_ld();
-#pragma unroll
-            for (int cb = 0; cb < 32; cb += 8) {
-                uint32_t w[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    w[e] = bias_act2_tc(v[cb + 2 * e], v[cb + 2 * e + 1], S.b1[c0 + cb + 2 * e], S.b1[c0 + cb + 2 * e + 1]);
-                *reinterpret_cast<uint4*>(S.h1 + canon(row, c0 + cb, TM)) = make_uint4(w[0], w[1], w[2], w[3]);
-            }
-        }
-        tr_publish();
-        // Z2 = H1 W2^T, H2 = tanh(Z2 + b2)
-        if (threadIdx.x == 0) mma_k(tm + TC_ACC, kdesc(su32(S.h1), TM), kstep(TM), kdesc(su32(S.w2), HID), kstep(HID),
-                                    idesc(TM, HID), HID / 16);
-        ok = tr_sync_mma(S, ph, err);
+        if (leader) mma_k(tm + TC_ACC, kdesc(su32(S.x), TM), kstep(TM), kdesc(su32(W.w1), HID), kstep(HID),
+                          idesc(TM, HID), KX_TC / 16);
+        ok = tr_sync_mma<G>(S, g, leader, ph, err);
     }
     if (ok) {
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int c0 = 64 * half + 32 * q;
-            uint32_t v[32];
-            tmem_ld32(tl + TC_ACC + (uint32_t)c0, v);
-            tmem_wait_ld();
-#pragma unroll
-            for (int cb = 0; cb < 32; cb += 8) {
-                uint32_t w[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    w[e] = bias_act2_tc(v[cb + 2 * e], v[cb + 2 * e + 1], S.b2[c0 + cb + 2 * e], S.b2[c0 + cb + 2 * e + 1]);
-                *reinterpret_cast<uint4*>(S.h2 + canon(row, c0 + cb, TM)) = make_uint4(w[0], w[1], w[2], w[3]);
-            }
-        }
-        tr_publish();
+        tanh_forward<G>(S.h1, tl + TC_ACC, W.b1, row, c0);
+        tr_publish<G>(g);
+        // Z2 = H1 W2^T, H2 = tanh(Z2 + b2)
+        if (leader) mma_k(tm + TC_ACC, kdesc(su32(S.h1), TM), kstep(TM), kdesc(su32(W.w2), HID), kstep(HID),
+                                    idesc(TM, HID), HID / 16);
+        ok = tr_sync_mma<G>(S, g, leader, ph, err);
+    }
+    if (ok) {
+        tanh_forward<G>(S.h2, tl + TC_ACC, W.b2, row, c0);
+        tr_publish<G>(g);
         // Y = H2 W3^T (+ b3 below)
-        if (threadIdx.x == 0) mma_k(tm + TC_ACC, kdesc(su32(S.h2), TM), kstep(TM), kdesc(su32(S.w3), OUTP), kstep(OUTP),
+        if (leader) mma_k(tm + TC_ACC, kdesc(su32(S.h2), TM), kstep(TM), kdesc(su32(W.w3), OUTP), kstep(OUTP),
                                     idesc(TM, OUTP), HID / 16);
-        ok = tr_sync_mma(S, ph, err);
+        ok = tr_sync_mma<G>(S, g, leader, ph, err);
     }
     if (ok) {
         // dY = 2 (y - t) / (B 9) on the tile's samples and the 9 outputs, else 0;
-        // the loss and b3's gradient (column sums of the BF16 dY) per warp
+        // the loss and b3's gradient (column sums of the BF16 dY) per warp,
+        // summed while the next contractions run
         const float inv = 2.f / (float)(B * NOUT);
-        if (half == 0) {
+        float lsum = 0.f;
+        uint32_t w[OUTP / 2];
+        if (share == 0) {
             uint32_t v[16];
             tmem_ld16(tl + TC_ACC, v);
             tmem_wait_ld();
             const bool valid = row0 + row < B;
-            float lsum = 0.f, d[OUTP];
+            float d[OUTP];
 #pragma unroll
             for (int o = 0; o < OUTP; ++o) {
                 d[o] = 0.f;
                 if (valid && o < NOUT) {
-                    const float rr = __uint_as_float(v[o]) + S.b3[o] - tgt[o];
+                    const float rr = __uint_as_float(v[o]) + W.b3[o] - tgt[o];
                     lsum += rr * rr;
                     d[o] = inv * rr;
                 }
             }
-            uint32_t w[OUTP / 2];
 #pragma unroll
             for (int e = 0; e < OUTP / 2; ++e) w[e] = pack_bf16_tc(d[2 * e], d[2 * e + 1]);
             *reinterpret_cast<uint4*>(S.dy + canon(row, 0, TM)) = make_uint4(w[0], w[1], w[2], w[3]);
             *reinterpret_cast<uint4*>(S.dy + canon(row, 8, TM)) = make_uint4(w[4], w[5], w[6], w[7]);
+        }
+        tr_publish<G>(g);
+        // dH2 = dY W3 (K = 16 outputs; W3 read MN-major) and dW3^T = H2^T dY
+        // (M = inputs, N = outputs, K = samples; both read MN-major)
+        if (leader) {
+            mma_k(tm + TC_ACC, kdesc(su32(S.dy), TM), kstep(TM), mdesc(su32(W.w3), OUTP), MSTEP, idesc_t(TM, HID, 0, 1), 1);
+            mma_k(tm + TC_DW3, mdesc(su32(S.h2), TM), MSTEP, mdesc(su32(S.dy), TM), MSTEP, idesc_t(HID, OUTP, 1, 1),
+                  TM / 16);
+        }
+        __syncwarp();
+        if (share == 0) {
 #pragma unroll
             for (int o = 0; o < NOUT; ++o) {
                 const __nv_bfloat162 pr = *reinterpret_cast<const __nv_bfloat162*>(&w[o / 2]);
@@ -983,93 +1023,87 @@ __global__ void __launch_bounds__(TR_THREADS, 1) k_loss_grad_tc(const float* __r
             for (int sh = 16; sh > 0; sh >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, sh);
             if (lane == 0) S.wloss[quarter] = lsum / (float)(B * NOUT);
         }
-        tr_publish();
-        // dH2 = dY W3 (K = 16 outputs; W3 read MN-major) and dW3^T = H2^T dY
-        // (M = inputs, N = outputs, K = samples; both read MN-major)
-        if (threadIdx.x == 0) {
-            mma_k(tm + TC_ACC, kdesc(su32(S.dy), TM), kstep(TM), mdesc(su32(S.w3), OUTP), MSTEP, idesc_t(TM, HID, 0, 1), 1);
-            mma_k(tm + TC_DW3, mdesc(su32(S.h2), TM), MSTEP, mdesc(su32(S.dy), TM), MSTEP, idesc_t(HID, OUTP, 1, 1),
-                  TM / 16);
-        }
-        ok = tr_sync_mma(S, ph, err);
+        ok = tr_sync_mma<G>(S, g, leader, ph, err);
     }
     if (ok) {
-        // dZ2 = dH2 (1 - H2^2) over H2; dW3 from its transpose (lane = input)
-        tanh_backward(S.h2, tl + TC_ACC, row, 64 * half);
-        if (half == 1) {
-            uint32_t v[16];
-            tmem_ld16(tl + TC_DW3, v);
+        // dZ2 = dH2 (1 - H2^2) over H2
+        tanh_backward<G>(S.h2, tl + TC_ACC, row, c0);
+        uint32_t w3[16];
+        if (share == 1) {
+            tmem_ld16(tl + TC_DW3, w3);
             tmem_wait_ld();
-#pragma unroll
-            for (int o = 0; o < NOUT; ++o) out[OFF_W3 + o * HID + row] = __uint_as_float(v[o]);
         }
-        tr_publish();
-        // dH1 = dZ2 W2 (W2 read MN-major) and dW2 = dZ2^T [H1 | 1]
-        // (M = outputs, N = inputs and the ones column, K = samples)
-        if (threadIdx.x == 0) {
-            mma_k(tm + TC_ACC, kdesc(su32(S.h2), TM), kstep(TM), mdesc(su32(S.w2), HID), MSTEP, idesc_t(TM, HID, 0, 1),
+        tr_publish<G>(g);
+        // dH1 = dZ2 W2 (W2 read MN-major) and dW2 = dZ2^T H1
+        // (M = outputs, N = inputs, K = samples)
+        if (leader) {
+            mma_k(tm + TC_ACC, kdesc(su32(S.h2), TM), kstep(TM), mdesc(su32(W.w2), HID), MSTEP, idesc_t(TM, HID, 0, 1),
                   HID / 16);
-            mma_k(tm + TC_DW2, mdesc(su32(S.h2), TM), MSTEP, mdesc(su32(S.h1), TM), MSTEP, idesc_t(HID, H1K, 1, 1),
+            mma_k(tm + TC_DW2, mdesc(su32(S.h2), TM), MSTEP, mdesc(su32(S.h1), TM), MSTEP, idesc_t(HID, HID, 1, 1),
                   TM / 16);
         }
-        ok = tr_sync_mma(S, ph, err);
+        // dW3 from its transpose (lane = input)
+        if (share == 1) {
+#pragma unroll
+            for (int o = 0; o < NOUT; ++o) out[OFF_W3 + o * HID + row] = __uint_as_float(w3[o]);
+        }
+        ok = tr_sync_mma<G>(S, g, leader, ph, err);
     }
     if (ok) {
-        // dZ1 = dH1 (1 - H1^2) over H1's first 128 columns; dW2 and b2's gradient
-        tanh_backward(S.h1, tl + TC_ACC, row, 64 * half);
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int c0 = 64 * half + 32 * q;
-            uint32_t v[32];
-            tmem_ld32(tl + TC_DW2 + (uint32_t)c0, v);
-            tmem_wait_ld();
-#pragma unroll
-            for (int e = 0; e < 32; ++e) out[OFF_W2 + row * HID + c0 + e] = __uint_as_float(v[e]);
-        }
-        if (half == 0) {
-            uint32_t v[16];
-            tmem_ld16(tl + TC_DW2 + (uint32_t)ONES_H, v);
-            tmem_wait_ld();
-            out[OFF_B2 + row] = __uint_as_float(v[0]);
-        }
-        tr_publish();
-        // dW1 = dZ1^T [X | 1] (M = outputs, N = the 48 input columns, K = samples)
-        if (threadIdx.x == 0)
+        // dZ1 = dH1 (1 - H1^2) over H1's first 128 columns
+        tanh_backward<G>(S.h1, tl + TC_ACC, row, c0);
+        tr_publish<G>(g);
+        // dW1 = dZ1^T [X | 1] (M = outputs, N = the 48 input columns, K = samples) and b2's
+        // gradient dZ2^T 1 (H1's ones column and the zeros behind it)
+        if (leader) {
             mma_k(tm + TC_DW1, mdesc(su32(S.h1), TM), MSTEP, mdesc(su32(S.x), TM), MSTEP, idesc_t(HID, KX_TC, 1, 1),
                   TM / 16);
-        ok = tr_sync_mma(S, ph, err);
+            mma_k(tm + TC_DB2, mdesc(su32(S.h2), TM), MSTEP, mdesc(su32(S.h1 + canon(0, ONES_H, TM)), TM), MSTEP,
+                  idesc_t(HID, H1K - HID, 1, 1), TM / 16);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int c = c0; c < c0 + COLS; c += 32) {
+            uint32_t v[32];
+            tmem_ld32(tl + TC_DW2 + (uint32_t)c, v);
+            tmem_wait_ld();
+#pragma unroll
+            for (int e = 0; e < 32; ++e) out[slot_w2(row, c + e)] = __uint_as_float(v[e]);
+        }
+        ok = tr_sync_mma<G>(S, g, leader, ph, err);
     }
     if (ok) {
-        if (half == 0) {
-            uint32_t v[32];
-            tmem_ld32(tl + TC_DW1, v);
-            tmem_wait_ld();
+        // dW1 and b1's gradient behind it, b2's: 16 columns at a time
 #pragma unroll
-            for (int e = 0; e < 32; ++e) out[OFF_W1 + row * NIN + e] = __uint_as_float(v[e]);
-        } else {
+        for (int c = 16 * share; c <= (int)TC_DB2; c += 16 * (GT / TM)) {
             uint32_t v[16];
-            tmem_ld16(tl + TC_DW1 + 32u, v);
+            tmem_ld16(tl + TC_DW1 + (uint32_t)c, v);
             tmem_wait_ld();
 #pragma unroll
-            for (int e = 0; e < NIN - 32; ++e) out[OFF_W1 + row * NIN + 32 + e] = __uint_as_float(v[e]);
-            out[OFF_B1 + row] = __uint_as_float(v[ONES_X - 32]);
+            for (int e = 0; e < 16; ++e) {
+                if (c + e < NIN) out[slot_w1(row, c + e)] = __uint_as_float(v[e]);
+                if (c + e == ONES_X) out[OFF_B1 + row] = __uint_as_float(v[e]);
+                if (c + e == (int)TC_DB2) out[OFF_B2 + row] = __uint_as_float(v[e]);
+            }
         }
-        if (threadIdx.x < NOUT) {
-            float c = 0.f;
-            for (int q = 0; q < GWARPS; ++q) c += S.wb3[q][threadIdx.x];
-            out[OFF_B3 + threadIdx.x] = c;
-        }
-        if (threadIdx.x == 0) {
-            float l = 0.f;
-            for (int q = 0; q < GWARPS; ++q) l += S.wloss[q];
-            out[NPARAM] = l;
+        if (share == 1 && quarter == 0) {
+            if (lane < NOUT) {
+                float c = 0.f;
+                for (int q = 0; q < GWARPS; ++q) c += S.wb3[q][lane];
+                out[OFF_B3 + lane] = c;
+            }
+            if (lane == 0) {
+                float l = 0.f;
+                for (int q = 0; q < GWARPS; ++q) l += S.wloss[q];
+                out[NPARAM] = l;
+            }
         }
     }
     fence_before();
     __syncthreads();
-    if (warp == 0) {
+    if (threadIdx.x < 32) {
         fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(S.tmem), "r"(TMEM_COLS) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(W.tmem), "r"(TR_COLS * G) : "memory");
     }
 }
 
@@ -1116,14 +1150,25 @@ int loss_grad_tc(const float* X, const float* T, const int* idx, long B, const P
                  void* stream) {
     static bool attr = false;
     if (!attr) {
-        if (cudaFuncSetAttribute(k_loss_grad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrSmem)) !=
-            cudaSuccess)
+        if (cudaFuncSetAttribute(k_loss_grad_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrSmem<1>)) !=
+                cudaSuccess ||
+            cudaFuncSetAttribute(k_loss_grad_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrSmem<2>)) !=
+                cudaSuccess)
             return -4;
         attr = true;
     }
-    const long blocks = (B + TM - 1) / TM;
-    k_loss_grad_tc<<<(unsigned)blocks, TR_THREADS, sizeof(TrSmem), (cudaStream_t)stream>>>(X, T, idx, B, P, part, err);
-    return cudaGetLastError() == cudaSuccess ? 0 : -4;
+    const long tiles = (B + TM - 1) / TM;
+    cudaError_t e;
+    // one tile per CTA while each gets an SM of its own; beyond, two.  Loss and
+    // gradient of 235 tiles 45.6 us with one, 41.3 with two, of 782 tiles 117
+    // and 98; a pair takes 1.5 times as long as a tile alone
+    if (tiles > sms_tc())
+        e = launch_pdl(k_loss_grad_tc<2>, dim3((unsigned)((tiles + 1) / 2)), dim3(TR_THREADS), sizeof(TrSmem<2>),
+                       (cudaStream_t)stream, true, X, T, idx, B, P, part, err);
+    else
+        e = launch_pdl(k_loss_grad_tc<1>, dim3((unsigned)tiles), dim3(TR_THREADS), sizeof(TrSmem<1>),
+                       (cudaStream_t)stream, true, X, T, idx, B, P, part, err);
+    return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? 0 : -4;
 }
 
 int forward_tc(const float* X, long M, const Packed* P, float* Y, int* err, void* stream) {
