@@ -496,7 +496,10 @@ __device__ __forceinline__ void consume(const Params& prm, int K, int sxK, int s
         int cls = -1;
         f2 aL[RB], bL[RB];                              // decay pairs (a, b) of the outputs being finalised
         f2 W[RB];                                       // sum of the target being completed
-        // the stage's barrier and its release
+        // The stage's barrier and its release, which follows the stores of what the stage's values went into:
+        // a load from the ring that is merely issued can be passed by the arrival, and the next box (async
+        // proxy) then lands before it reads.  (Released at once, one half-warp of one row in 10^6 stages read
+        // the next round's values on 1501 x 1099 cells; a proxy fence instead costs 3 % of a P_13 pass.)
         auto wait = [&]() -> bool { return wait_warp(base + 8 * r, ph, abort_flag, prm.err); };
         auto release = [&]() {
             arrive_warp(base + 8 * (MAX_STAGES + r), lane);
@@ -582,7 +585,6 @@ __device__ __forceinline__ void consume(const Params& prm, int K, int sxK, int s
             const uint32_t t = ring + r * S::STAGE_BYTES;
             differences(t, dx, dy);
             each_row([&](auto i) { u[i] = ld8<4 * i * TX>(t + ou); }, ROWS);
-            release();
 #pragma unroll
             for (int i = 0; i < RB; ++i) {
                 W[i] = f2_fma(w[0], dx[i], W[i]);
@@ -595,6 +597,7 @@ __device__ __forceinline__ void consume(const Params& prm, int K, int sxK, int s
                 W[i] = ld8<i * PI>(pq);
                 st8<i * PI>(pq, Nn[i]);
             }, ROWS);
+            release();
             return true;
         };
         if (first == 1)                         // the even pass completes order 0 after order 1 alone: no partial sums yet
@@ -626,12 +629,12 @@ __device__ __forceinline__ void consume(const Params& prm, int K, int sxK, int s
                 rec += S::REC_BYTES;
                 if (!wait()) return;
                 differences(ring + r * S::STAGE_BYTES, dx, dy);
-                release();
                 each_row([&](auto i) {
                     Nn[i] = f2_fma(w[3], dy[i], f2_fma(w[2], dx[i], zero2()));
                     W[i] = ld8<i * PI>(pq);
                     st8<i * PI>(pq, Nn[i]);
                 }, ROWS);
+                release();
                 for (int q = nq_of(lp) - 1; q > 0; --q) {
                     pq += PQ;
                     if (!full_step(pq, dx, dy)) return;
@@ -658,8 +661,8 @@ __device__ __forceinline__ void consume(const Params& prm, int K, int sxK, int s
                 if (!wait()) return;
                 const uint32_t t = ring + r * S::STAGE_BYTES;
                 each_row([&](auto i) { u[i] = ld8<4 * i * TX>(t + ou); }, ROWS);
-                release();
                 if (__any_sync(0xffffffffu, f.x >= 0)) finalise(f, u);
+                release();
                 pq += PQ;
                 if (body) {
                     if (lp < N) each_row([&](auto i) { st8<i * PI>(pq, Nn[i]); }, ROWS);
