@@ -89,7 +89,7 @@ constexpr int WIDE_BAND_MAX_N = 15;
 // kernels.
 struct Variant {
     int ty, byi, threads, part_bytes, stage_bytes, rec_bytes, minb;
-    void (*pass)(Params, int);
+    void (*pass[2])(Params, int);         // [WARM]
     void (*batch)(const Params*, const int4*, const int*, int, int);
 };
 // 10-row tiles as two bands of five rows, two CTAs per SM: the fewest
@@ -106,7 +106,7 @@ struct Variant {
 enum { TALL_WIDE, TALL, TALL_LEAN, SHORT, SHAPES };
 template <class S>
 Variant variant_of() {
-    return {S::TY, S::BYI, S::THREADS, S::PART_BYTES, S::STAGE_BYTES, S::REC_BYTES, S::MINB, k_tiled_pass<S>, k_tiled_batch<S>};
+    return {S::TY, S::BYI, S::THREADS, S::PART_BYTES, S::STAGE_BYTES, S::REC_BYTES, S::MINB, {k_tiled_pass<S, false>, k_tiled_pass<S, true>}, k_tiled_batch<S>};
 }
 const Variant kVariant[SHAPES] = {variant_of<Shape<5, 2, 2, true>>(), variant_of<Shape<2, 5, 1, true>>(),
                                   variant_of<Shape<2, 5, 1, false>>(), variant_of<Shape<1, 5, 2, true>>()};
@@ -606,10 +606,11 @@ int tiled_update(TiledPlan* pl, const SystemMatrices& sys, const std::vector<int
         const int stage_off = tables;
         tables += (int)(t.stages.size() * sizeof(int4));
         const int ring_off = (tables + 127) & ~127;
-        int dev = 0, maxsm = 0, persm = 0;
+        int dev = 0, maxsm = 0, persm = 0, l2 = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
         cudaDeviceGetAttribute(&persm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+        cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
         // per-CTA budget at c CTAs per SM (1 KB reserved per CTA), less the
         // batch kernel's static parameter copy
         auto ring_for = [&](int c) {
@@ -625,11 +626,11 @@ int tiled_update(TiledPlan* pl, const SystemMatrices& sys, const std::vector<int
         pl->smem_bytes[P] = ring_off + nring * V.stage_bytes;
         pl->nring[P] = nring;
         // (the function's limit, common to every handle: not this plan's need)
-        const cudaError_t fe = cudaFuncSetAttribute(V.pass, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm);
-        if (fe != cudaSuccess) {
-            pl->err = "cudaFuncSetAttribute failed";
-            return -4;
-        }
+        for (auto pass : V.pass)
+            if (cudaFuncSetAttribute(pass, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm) != cudaSuccess) {
+                pl->err = "cudaFuncSetAttribute failed";
+                return -4;
+            }
         for (int w = 0; w < 2; ++w) {
             Params& prm = pl->prm[P][w];
             std::memset(&prm, 0, sizeof(prm));
@@ -664,11 +665,13 @@ int tiled_update(TiledPlan* pl, const SystemMatrices& sys, const std::vector<int
             prm.err = pl->err_dev;
             prm.smem_stage_off = stage_off;
             prm.smem_ring_off = ring_off;
+            int nsrc[2] = {0, 0};
             for (int K = 0; K < 2; ++K) {
                 unsigned long long src = 0;
                 bool one = true;
                 for (const int4& f : fk[K])
                     if ((f.z | f.w) != 0) {
+                        ++nsrc[K];
                         const unsigned long long a = ((unsigned long long)(unsigned)f.w << 32) | (unsigned)f.z;
                         if (src != 0 && a != src) one = false;
                         src = a;
@@ -676,6 +679,13 @@ int tiled_update(TiledPlan* pl, const SystemMatrices& sys, const std::vector<int
                 prm.any_src[K] = src != 0;
                 prm.pf_src[K] = one ? (const float*)(uintptr_t)src : nullptr;
             }
+            // The variant that warms L1 (WARM) pays where the consumers load a source for most targets and L2
+            // does not hold them beside the state: P_9 on 512^2 (116 MB) 12 % of a pass, P_39 on 150^2 (150 MB)
+            // 42 %; P_13 on 200^2 (34 MB) loses 2 %, a pass with a single source 4 %.
+            long bytes = 0;
+            for (int g = 0; g < 4; ++g) bytes += (long)pl->geo.K[g] * pl->geo.cstride[g] * 4;
+            for (int K = 0; K < 2; ++K) bytes += 2l * nsrc[K] * prm.out[K].cp * prm.out[K].ny * 4;  // (both passes' alike)
+            prm.many_src = nsrc[0] + nsrc[1] >= prm.nstages && bytes > l2 / 2;
         }
     }
     pl->ready = true;
@@ -762,7 +772,8 @@ int tiled_pass(TiledPlan* pl, bool odd, int which, void* stream) {
     const bool pdl = tiled_overlap(pl, odd);
     cudaError_t e;
     const Variant& V = kVariant[pl->shape];
-    e = launch_pdl(V.pass, dim3(grid), dim3(V.threads), (size_t)pl->smem_bytes[P],
+    const Params& prm = pl->prm[P][which];
+    e = launch_pdl(V.pass[prm.many_src], dim3(grid), dim3(V.threads), (size_t)pl->smem_bytes[P],
                    (cudaStream_t)stream, pdl, pl->prm[P][which], ntiles);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {

@@ -102,7 +102,7 @@ constexpr int MAXN = 63;
 // sums; tables; ring.  (A step may read one q past the partial sums: table
 // values that nothing uses.)
 constexpr int PART_OFF = 256;
-static_assert(2 * MAX_STAGES * 8 + 4 <= PART_OFF, "barriers fit before the partial sums");
+static_assert(2 * MAX_STAGES * 8 + 4 <= PART_OFF - 8, "barriers fit before the scratch word and the partial sums");
 constexpr unsigned long long WAIT_NS = 2000000000ull;   // bounded waits: 2 s
 
 struct OutGrid {
@@ -136,6 +136,7 @@ struct Params {
     int* err;                   // bounded-wait failure flag
     int smem_rec_off[2], smem_stage_off, smem_ring_off;     // byte offsets in dynamic smem
     int any_src[2];             // per output kind: whether any finalised component has a source
+    int many_src;               // whether half of the targets or more have one
     const float* pf_src[2];     // per output kind: the source array its finalisations read, if it
                                 // has exactly one (prefetched into L2 with the decay pairs), else null
 };
@@ -680,6 +681,12 @@ __device__ __forceinline__ void consume(const Params& prm, int K, int sxK, int s
     }
 }
 
+// The 32 bytes at a into L1: a 4-byte copy to a word that nothing reads
+// (prefetch.global.L1 brought half the gain).
+__device__ __forceinline__ void warm_line(const float* a, uint32_t scratch) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(scratch), "l"(a) : "memory");
+}
+
 // Tiles t0, t0 + tstride, ... < tend of one pass, through one continuous
 // pipeline: the producer walks a global stage index over all of them (the
 // first stages of the next tile are in flight while the consumers finish
@@ -688,7 +695,7 @@ __device__ __forceinline__ void consume(const Params& prm, int K, int sxK, int s
 // reads them from there); prm: everything else.  first_call: the CTA's
 // first call (a later call invalidates and re-initialises the barriers; the
 // caller synchronises the CTA in between).
-template <class S>
+template <class S, bool WARM>
 __device__ __forceinline__ void tiled_tiles(const Params& prm, const CUtensorMap* maps, int t0, int tstride, int tend,
                                             bool first_call) {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -772,6 +779,22 @@ __device__ __forceinline__ void tiled_tiles(const Params& prm, const CUtensorMap
     const int nst = prm.nstages;
     int r = 0, u = 0, issued = 0;
     bool ok = true;
+    // The output warp also has the values that the consumers load one by one
+    // (a source of every target, the decay pairs of every order) brought into
+    // L1, a ring of stages before they are used: such a load stood in the
+    // chain of steps with its whole latency.  150^2 P_39 with both: 168 us per
+    // pass without, 115 with (prefetch.global.L1 instead of the copies: 128;
+    // loads into registers a step or two ahead, in the consumers: 174 to 179).
+    // WARM: the output warp also has the values that the consumers load one by
+    // one (a source of every target, the decay pairs of every order) brought
+    // into L1, a ring of stages before they are used.
+    const uint32_t scratch = base + PART_OFF - 8;
+    // A row of 64 values at any alignment: 9 x 32 bytes, or, for the tiles of ten rows, which leave L1 little
+    // room, 3 x 128 (whose other sectors then come from L2).  us per pass, none / 9 / 3: 150^2 P_39 164 / 98 to 103
+    // / 114, 300^2 331 / 237 / 220, 512^2 P_9 42 / 40 / 38.  (Loads into registers a step or two ahead, by the
+    // consumers: 174 to 179; prefetch.global.L1: 128.)
+    constexpr int STEP = S::RB == 1 ? 8 : 32, PER = TX / STEP + 1;
+    constexpr int LINES = (PER * S::TY + 31) / 32;
     for (int tl = 0; tl < ntl && ok; ++tl) {
         // box origins (tensor coordinates x' = x + VEC, row = y + 1)
         const int tile = t0 + tl * tstride;
@@ -780,6 +803,17 @@ __device__ __forceinline__ void tiled_tiles(const Params& prm, const CUtensorMap
         const int bxR = h == 0 ? x0 + (sxR == 0 ? 0 : VEC) : x0 + VEC, byR = h == 0 ? y0 + (syR == 0 ? 0 : 1) : y0 + 1;
         const int bxI = h == 0 ? x0 + (sxI == 0 ? 0 : VEC) : x0 + VEC, byI = h == 0 ? y0 + (syI == 0 ? 0 : 1) : y0 + 1;
         int k = 0;
+        int order_at = 0, next = 1 - prm.P;             // the stage at which input order `next` starts
+        int line[2][LINES];                             // the lane's 32 bytes of the tile's rows from row y0 on, per kind
+        if constexpr (WARM)
+#pragma unroll
+            for (int kind = 0; kind < 2; ++kind)
+#pragma unroll
+                for (int j = 0; j < LINES; ++j) {
+                    const OutGrid& Gk = prm.out[kind];
+                    const int e = lane + 32 * j, row = min(min(e / PER, S::TY - 1), Gk.ny - 1 - y0);
+                    line[kind][j] = row * Gk.cp + min(x0 + min(STEP * (e % PER), TX - 1), Gk.cp - 1);
+                }
         auto issue = [&](int kend) {
             for (; k < kend && ok; ++k) {
                 const int2 c = s_comp[2 * k];
@@ -792,6 +826,31 @@ __device__ __forceinline__ void tiled_tiles(const Params& prm, const CUtensorMap
                     expect_tx(bar, ((c.x >= 0 ? 1u : 0u) + (c.y >= 0 ? 1u : 0u)) * box_bytes);
                     if (c.x >= 0) tma_box(dst + oR, mR, bxR, byR, c.x, bar);
                     if (c.y >= 0) tma_box(dst + oI, mI, bxI, byI, c.y, bar);
+                }
+                if constexpr (WARM) if (h == 1) {
+                    auto warm = [&](const float* a, int kind) {
+#pragma unroll
+                        for (int j = 0; j < LINES; ++j)
+                            warm_line(a + (long)y0 * prm.out[kind].cp + line[kind][j], scratch);
+                    };
+                    // input order `next` starts here: the decay pairs of the target order below it
+                    if (k == order_at) {
+                        if (next > 0 && prm.nclasses != 2 && prm.out[0].coef != nullptr && prm.out[1].coef != nullptr)
+#pragma unroll
+                            for (int kind = 0; kind < 2; ++kind) {
+                                const long plane = (long)prm.out[kind].cp * prm.out[kind].ny;
+                                const float* ca = prm.out[kind].coef + ((long)(next - 1) * 4 + 2 * prm.which) * plane;
+                                warm(ca, kind);
+                                warm(ca + plane, kind);
+                            }
+                        order_at += next <= prm.N ? nq_of(next) + (next & 1) : nst;
+                        next += 2;
+                    }
+#pragma unroll
+                    for (int kind = 0; kind < 2; ++kind) {
+                        const int4 f = ld16i(base + prm.smem_rec_off[kind] + (k + 1) * S::REC_BYTES - 16);
+                        if (__any_sync(0xffffffffu, (f.z | f.w) != 0)) warm(source_of(f), kind);
+                    }
                 }
                 ++issued;
                 if (++r == NR) { r = 0; ++u; }
@@ -819,6 +878,7 @@ __device__ __forceinline__ void tiled_tiles(const Params& prm, const CUtensorMap
         }
         issue(nst);
     }
+    if constexpr (WARM) asm volatile("cp.async.wait_all;" ::: "memory");
     if (!ok && lane == 0) {
         // aborted: wait (bounded) for the copies still in flight
         for (int G = issued - 1; G >= 0 && G > issued - 1 - NR; --G) {
@@ -833,10 +893,10 @@ __device__ __forceinline__ void tiled_tiles(const Params& prm, const CUtensorMap
 // ... (raster order).  The CTAs then work on one contiguous band of tiles
 // at any time, so the halo rows that vertically adjacent tiles share come
 // from DRAM once, and each CTA's pipeline runs on across its tiles.
-template <class S>
+template <class S, bool WARM>
 __global__ void __launch_bounds__(S::THREADS, S::MINB) k_tiled_pass(const __grid_constant__ Params prm,
                                                                                     int ntiles) {
-    tiled_tiles<S>(prm, prm.maps, blockIdx.x, gridDim.x, ntiles, true);
+    tiled_tiles<S, WARM>(prm, prm.maps, blockIdx.x, gridDim.x, ntiles, true);
 }
 
 // Batched pass: CTA b runs items[off[b]] .. items[off[b + 1] - 1], each a
@@ -862,7 +922,7 @@ __global__ void __launch_bounds__(S::THREADS, S::MINB) k_tiled_batch(const Param
             for (int i = threadIdx.x; i < (int)(sizeof(Params) / 16); i += blockDim.x) dst[i] = src[i];
         }
         __syncthreads();
-        tiled_tiles<S>(s_prm, g->maps, item.y, item.w, item.y + (item.z - 1) * item.w + 1, it == begin);
+        tiled_tiles<S, false>(s_prm, g->maps, item.y, item.w, item.y + (item.z - 1) * item.w + 1, it == begin);
     }
 }
 

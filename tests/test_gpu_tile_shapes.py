@@ -95,3 +95,25 @@ def test_runs_repeat_bit_for_bit():
         got = s.get_state()
         assert ref is None or got == ref
         ref = got
+
+
+def test_sources_in_every_moment():
+    """A source in every moment and a decay class per order, on a state that
+    L2 does not hold beside its sources (the kernels that load them into L1
+    ahead): 10-row and 5-row tiles bit for bit, and the gather kernel at the
+    FP32 parity bar."""
+    from helpers import assert_parity
+    from test_gpu_parity import FP32_TOL
+    N, n = 35, (161, 137)
+    p = _random_problem(N, n, ("periodic", "extrapolation"), "fp32", 990, 2, aniso=True)
+    got = []
+    for kernel in ("tiled_tall", "tiled_short", "gather"):
+        s = capi.Stepper.from_problem(p, kernel=kernel, schedule="merged")
+        for j in range(s.ncomp):
+            X, Y = s.grid_coords(s.moment_info(j)["grid"])
+            s.set_source(j, np.cos(0.7 * j + 3 * X) * np.exp(-Y) / (1 + j % 7))
+        s.step(2)
+        got.append([s.moments(j) for j in range(s.ncomp)])
+    for a, b in zip(got[0], got[1]):
+        assert np.array_equal(a, b)
+    assert_parity(got[0], [np.asarray(a, np.float64) for a in got[2]], FP32_TOL, "fp32")
