@@ -681,7 +681,7 @@ int tiled_update(TiledPlan* pl, const SystemMatrices& sys, const std::vector<int
             }
             // The variant that warms L1 (WARM) pays where the consumers load a source for most targets and L2
             // does not hold them beside the state: P_9 on 512^2 (116 MB) 12 % of a pass, P_39 on 150^2 (150 MB)
-            // 42 %; P_13 on 200^2 (34 MB) loses 2 %, a pass with a single source 4 %.
+            // 37 %; P_13 on 200^2 (34 MB) loses 2 %, a pass with a single source 4 %.
             long bytes = 0;
             for (int g = 0; g < 4; ++g) bytes += (long)pl->geo.K[g] * pl->geo.cstride[g] * 4;
             for (int K = 0; K < 2; ++K) bytes += 2l * nsrc[K] * prm.out[K].cp * prm.out[K].ny * 4;  // (both passes' alike)
