@@ -511,8 +511,12 @@ __device__ __forceinline__ void fused_tiles(const FusedParams& prm, int t0, int 
                 const float* t = stage_ptr();
                 accumulate(t, Pc_, Pn_, Nc_, Nn_);
                 if (q >= 1 && q - 1 < nqp) finalize(t, Pc_);
+                // Before the slot's release: the store waits for both differences, and a load that is merely
+                // issued can be passed by the arrival, the next box then landing before it reads
+                // (tiled_kernel.cuh).  In the top input order, which has no next-order targets, entry q has
+                // been read for the last time, so every stage stores.
+                pp[q * ncons] = Nc_;
                 stage_done();
-                if (q < nqn) pp[q * ncons] = Nc_;
             };
             int q = 0;
             for (; q + 1 < nq && alive; q += 2) {
