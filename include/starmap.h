@@ -422,6 +422,11 @@ int starmap_sync(starmap_t* h);
  * usable).  STARMAP_E_STATE if a wait did not give up, STARMAP_E_CUDA if a
  * kernel could not run.  Synchronous (legacy default stream), about 8 s. */
 int starmap_selftest_bounded_wait(void);
+/* The clean-up after an expired wait: runs the end of a tiled pass's two
+ * producer warps that gave up three pipeline stages apart, and returns the
+ * microseconds it took in *us (each stage that one of them leaves half armed
+ * would be a wait of 2 s).  STARMAP_E_ARG, STARMAP_E_CUDA.  Synchronous (legacy default stream). */
+int starmap_selftest_abort_drain(int* us);
 
 /* Host-side fault injection for tests (no counterpart in the paper): the
  * n-th device allocation the library makes from now on (in any handle,

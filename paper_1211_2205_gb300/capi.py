@@ -136,6 +136,7 @@ def lib():
         "starmap_unpack_rows": (ctypes.c_int, [H, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_void_p,
                                                ctypes.c_size_t]),
         "starmap_selftest_bounded_wait": (ctypes.c_int, []),
+        "starmap_selftest_abort_drain": (ctypes.c_int, [ctypes.POINTER(ctypes.c_int)]),
         "starmap_diagnostics_noalloc": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_int,
                                                        ctypes.c_int, ctypes.c_long, ctypes.c_long, ctypes.c_long,
                                                        ctypes.c_double, ctypes.c_void_p, ctypes.c_void_p]),
@@ -276,6 +277,15 @@ def debug_fail_allocation(n: int) -> int:
 def selftest_bounded_wait() -> int:
     """Status of the bounded-wait self-test (E_TIMEOUT is the expected outcome)."""
     return lib().starmap_selftest_bounded_wait()
+
+
+def selftest_abort_drain() -> int:
+    """Microseconds the clean-up of two producer warps takes that gave up some stages apart."""
+    us = ctypes.c_int(-1)
+    rc = lib().starmap_selftest_abort_drain(ctypes.byref(us))
+    if rc != OK:
+        raise StarmapError(rc, lib().starmap_last_error(None).decode())
+    return us.value
 
 
 def health_verdict(l2_start: float, l2_end: float, t_span: float, q_l2: float, growth: float,

@@ -1464,6 +1464,12 @@ int starmap_selftest_bounded_wait(void) {
     return fail(nullptr, STARMAP_E_TIMEOUT, "bounded waits gave up as expected");
 }
 
+int starmap_selftest_abort_drain(int* us) {
+    if (!us) return fail(nullptr, STARMAP_E_ARG, "us is NULL");
+    if (tiled_drain_selftest(us)) return fail(nullptr, STARMAP_E_CUDA, "drain self-test could not run");
+    return STARMAP_OK;
+}
+
 int starmap_sync(starmap_t* h) {
     if (!h) return STARMAP_E_ARG;
     CK(cudaStreamSynchronize(h->stream), "sync");

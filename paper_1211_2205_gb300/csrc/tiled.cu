@@ -838,7 +838,42 @@ __global__ void k_wait_selftest(int* err, int* result) {
     __syncthreads();
     if (threadIdx.x == 0) *result = wait_bounded(&bar, 0, &abort_flag, err) ? 1 : 0;
 }
+// The end of two producer warps that gave up three stages apart (no boxes:
+// each stage is armed with no bytes): *result = microseconds the drain took.
+__global__ void k_drain_selftest(int* result) {
+    __shared__ uint64_t full[MAX_STAGES];
+    __shared__ int issued_by[PRODUCER_WARPS];
+    constexpr int NR = 4;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int r = 0; r < NR; ++r) mbar_init(&full[r], PRODUCER_WARPS);
+        for (int h = 0; h < PRODUCER_WARPS; ++h) issued_by[h] = -1;
+        fence_mbar_init();
+    }
+    __syncthreads();
+    // a whole ring by both, then three stages of the next round by the first alone
+    const int issued = warp == 0 ? NR + 3 : NR;
+    if (lane == 0)
+        for (int G = 0; G < NR; ++G) mbar_expect_tx(&full[G % NR], 0);
+    __syncthreads();
+    if (lane == 0)
+        for (int G = NR; G < issued; ++G) mbar_expect_tx(&full[G % NR], 0);
+    const unsigned long long t0 = global_ns();
+    if (lane == 0) drain(full, NR, issued_by, warp, issued);
+    __syncthreads();
+    if (threadIdx.x == 0) *result = (int)((global_ns() - t0) / 1000);
+}
 }  // namespace
+
+int tiled_drain_selftest(int* us) {
+    int* d = nullptr;
+    if (dev_alloc(&d, sizeof(int)) != cudaSuccess) return -4;
+    k_drain_selftest<<<1, 32 * PRODUCER_WARPS>>>(d);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpy(us, d, sizeof(int), cudaMemcpyDeviceToHost);
+    cudaFree(d);
+    return e == cudaSuccess ? 0 : -4;
+}
 
 int tiled_wait_selftest(int* gave_up) {
     int *d = nullptr;

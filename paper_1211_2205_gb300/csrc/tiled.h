@@ -68,6 +68,8 @@ int tiled_variant(TiledPlan* plan);
 // Self-test of the bounded wait (an mbarrier nothing arrives at); *gave_up = 1
 // when the wait expired and raised the flag as it must.
 int tiled_wait_selftest(int* gave_up);
+// Microseconds that the end of two producers takes that gave up some stages apart.
+int tiled_drain_selftest(int* us);
 // The tile shape of a batch's kernel: for a tile height and its highest order.
 int tiled_batch_shape(int variant, int max_N);
 // Resident CTAs per SM of that kernel with smem_bytes of dynamic shared memory.

@@ -98,11 +98,13 @@ struct Shape {
     static constexpr int REC_BYTES = DUP ? 80 : 48;                   // record of a stage and kind in shared memory
 };
 constexpr int MAXN = 63;
-// Shared memory: full[MAX_STAGES], empty[MAX_STAGES], abort flag; partial
-// sums; tables; ring.  (A step may read one q past the partial sums: table
-// values that nothing uses.)
+// Shared memory: full[MAX_STAGES], empty[MAX_STAGES], abort flag, the stages
+// each producer had issued when it gave up (drain), a scratch word (warm_line); partial sums;
+// tables; ring.  (A step may read one q past the partial sums: table values
+// that nothing uses.)
 constexpr int PART_OFF = 256;
-static_assert(2 * MAX_STAGES * 8 + 4 <= PART_OFF - 8, "barriers fit before the scratch word and the partial sums");
+constexpr int SCRATCH_OFF = PART_OFF - 4;
+static_assert(2 * MAX_STAGES * 8 + 4 * (1 + PRODUCER_WARPS) <= SCRATCH_OFF, "the barrier area");
 constexpr unsigned long long WAIT_NS = 2000000000ull;   // bounded waits: 2 s
 
 struct OutGrid {
@@ -681,6 +683,32 @@ __device__ __forceinline__ void consume(const Params& prm, int K, int sxK, int s
     }
 }
 
+// The end of a producer warp (h: which) that gave up after arming `issued`
+// stages.  The CTA must not leave, nor re-use its barriers, with copies in
+// flight, and a stage's full barrier needs both producers, of which one may
+// be ahead of the other by up to a ring.  So each waits for the other's count
+// (-1 until it gives up too), arrives, without a box, at what the other armed
+// alone, and waits for the last ring of stages, which now completes when its
+// copies land.  (The stages armed by one producer are of the current round:
+// it armed them after their slots had drained.)  One limit for all of it,
+// which a producer that had issued everything lets run out: its copies are
+// older than that then.  (A count from that one as well, stored at the end of
+// every pass, changed the code of the issuing loop: the beam's pass, 102 us,
+// took 1 to 2 % longer.)  The consumers' own waits end by the abort flag, or
+// with what has landed, in an error either way.
+__device__ __forceinline__ void drain(uint64_t* full, int NR, volatile int* issued_by, int h, int issued) {
+    static_assert(PRODUCER_WARPS == 2, "one other producer");
+    const unsigned long long t0 = global_ns();
+    issued_by[h] = issued;
+    while (issued_by[1 - h] < 0)
+        if (global_ns() - t0 > WAIT_NS) return;
+    const int all = max(issued, issued_by[1 - h]);
+    for (int G = issued; G < all; ++G) mbar_arrive(&full[G % NR]);
+    for (int G = max(0, all - NR); G < all; ++G)
+        while (!mbar_try_wait(&full[G % NR], (G / NR) & 1))
+            if (global_ns() - t0 > WAIT_NS) return;
+}
+
 // The 32 bytes at a into L1: a 4-byte copy to a word that nothing reads
 // (prefetch.global.L1 brought half the gain).
 __device__ __forceinline__ void warm_line(const float* a, uint32_t scratch) {
@@ -721,7 +749,7 @@ __device__ __forceinline__ void tiled_tiles(const Params& prm, const CUtensorMap
             mbar_init(&full[r], PRODUCER_WARPS);
             mbar_init(&empty[r], S::CONSUMER_WARPS);
         }
-        *abort_flag = 0;
+        for (int k = 0; k <= PRODUCER_WARPS; ++k) abort_flag[k] = k == 0 ? 0 : -1;      // and the stages issued
         fence_mbar_init();
     }
     // stage the records and the stage list in shared memory
@@ -788,7 +816,7 @@ __device__ __forceinline__ void tiled_tiles(const Params& prm, const CUtensorMap
     // WARM: the output warp also has the values that the consumers load one by
     // one (a source of every target, the decay pairs of every order) brought
     // into L1, a ring of stages before they are used.
-    const uint32_t scratch = base + PART_OFF - 8;
+    const uint32_t scratch = base + SCRATCH_OFF;
     // A row of 64 values at any alignment: 9 x 32 bytes, or, for the tiles of ten rows, which leave L1 little
     // room, 3 x 128 (whose other sectors then come from L2).  us per pass, none / 9 / 3: 150^2 P_39 164 / 98 to 103
     // / 114, 300^2 331 / 237 / 220, 512^2 P_9 42 / 40 / 38.  (Loads into registers a step or two ahead, by the
@@ -879,14 +907,7 @@ __device__ __forceinline__ void tiled_tiles(const Params& prm, const CUtensorMap
         issue(nst);
     }
     if constexpr (WARM) asm volatile("cp.async.wait_all;" ::: "memory");
-    if (!ok && lane == 0) {
-        // aborted: wait (bounded) for the copies still in flight
-        for (int G = issued - 1; G >= 0 && G > issued - 1 - NR; --G) {
-            const unsigned long long tw = global_ns();
-            while (!mbar_try_wait(&full[G % NR], (G / NR) & 1))
-                if (global_ns() - tw > WAIT_NS) break;
-        }
-    }
+    if (!ok && lane == 0) drain(full, NR, abort_flag + 1, h, issued);
 }
 
 // Single-instance pass: a persistent grid; CTA b takes tiles b, b + gridDim.x,

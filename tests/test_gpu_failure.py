@@ -20,3 +20,9 @@ def test_bounded_wait_gives_up_and_context_survives():
     o, ref = oracle_run(p, s)
     assert_parity(got, ref, 1e-5, "fp32")
     s.sync()
+
+
+def test_clean_up_after_an_abort_does_not_wait_for_the_other_producer():
+    """A stage that one producer armed and the other never will: the clean-up
+    completes it instead of waiting for its limit (2 s a stage)."""
+    assert 0 <= capi.selftest_abort_drain() < 500_000
