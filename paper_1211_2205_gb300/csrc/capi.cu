@@ -62,9 +62,10 @@ struct starmap_s {
     std::vector<double> sig_a[4], sig_s[4];
     std::vector<int> src_slot;            // per component, -1 if none
     std::vector<void*> src_dev;           // by slot
-    void* src_ptrs_dev = nullptr;
-    GatherOut* outs_dev = nullptr;
-    void* coefs_dev = nullptr;
+    DevTable src_ptrs_dev;
+    std::vector<GatherOut> outs;          // the gather kernel's outputs (empty where another kernel runs)
+    std::vector<int> outs_comp;           // and their components
+    DevTable outs_dev, coefs_dev;
     int tbeg[4] = {0, 0, 0, 0}, tend[4] = {0, 0, 0, 0};
     cudaStream_t stream = nullptr;
     bool own_stream = false;
@@ -78,6 +79,7 @@ struct starmap_s {
     int kernel_used = STARMAP_KERNEL_GATHER;
     TiledPlan* tiled = nullptr;
     StreamTables* stream64 = nullptr;     // FP64 2D passes (null: the gather kernel)
+    bool stream_tried = false;
     // learned closure (STARMAP_CLOSURE_MLP8)
     int closure = STARMAP_CLOSURE_NONE;
     int nsys = 0;                          // order of the assembled system
@@ -182,68 +184,82 @@ int class_of(const starmap_t* h, int l) {
     return l;
 }
 
-// Build the per-component pass tables (couplings, classes, source slots).
+// The gather kernel's tables (couplings once; classes, source slots).
+template <class T>
+int build_gather(starmap_t* h) {
+    const int n = h->ncomp;
+    if (h->outs.empty()) {
+        std::vector<GatherOut> outs;
+        std::vector<int> comps;
+        std::vector<GatherCoef<T>> coefs;
+        for (int g = 0; g < 4; ++g) {
+            h->tbeg[g] = (int)outs.size();
+            for (int j : h->members[g]) {
+                if (h->frozen[j]) continue;
+                GatherOut o{};
+                GatherCoef<T> c{};
+                o.local = h->sys.moms[j].local;
+                for (int k = 0; k < n; ++k) {
+                    double mx = h->sys.Mx[(size_t)j * n + k];
+                    double my = h->sys.My[(size_t)j * n + k];
+                    if (mx != 0.0) {
+                        if (h->sys.moms[k].grid != (g ^ 1) || o.nxt >= MAXC)
+                            return fail(h, STARMAP_E_UNSUPPORTED, "x-coupling outside the staggered pattern");
+                        o.xin[o.nxt] = h->sys.moms[k].local;
+                        c.cx[o.nxt] = (T)(-mx / h->dx);
+                        ++o.nxt;
+                    }
+                    if (my != 0.0) {
+                        if (h->sys.moms[k].grid != (g ^ 2) || o.nyt >= MAXC)
+                            return fail(h, STARMAP_E_UNSUPPORTED, "y-coupling outside the staggered pattern");
+                        o.yin[o.nyt] = h->sys.moms[k].local;
+                        c.cy[o.nyt] = (T)(-my / h->dy);
+                        ++o.nyt;
+                    }
+                }
+                outs.push_back(o);
+                comps.push_back(j);
+                coefs.push_back(c);
+            }
+            h->tend[g] = (int)outs.size();
+        }
+        CK(table_upload(h->coefs_dev, coefs.data(), coefs.size() * sizeof(GatherCoef<T>)), "cudaMalloc tables");
+        h->outs = outs;
+        h->outs_comp = comps;
+    }
+    for (size_t i = 0; i < h->outs.size(); ++i) {
+        h->outs[i].cls = h->comp_class[h->outs_comp[i]];
+        h->outs[i].src = h->src_slot[h->outs_comp[i]];
+    }
+    CK(table_upload(h->outs_dev, h->outs.data(), h->outs.size() * sizeof(GatherOut)), "cudaMalloc tables");
+    return STARMAP_OK;
+}
+
+// The pass tables of the handle's kernel.  What follows from the system alone
+// is assembled once; a source or a new set of decay classes changes the
+// entries' classes and source slots and uploads them into the same buffers.
 template <class T>
 int build_tables(starmap_t* h) {
-    std::vector<GatherOut> outs;
-    std::vector<GatherCoef<T>> coefs;
-    const int n = h->ncomp;
-    for (int g = 0; g < 4; ++g) {
-        h->tbeg[g] = (int)outs.size();
-        for (int j : h->members[g]) {
-            if (h->frozen[j]) continue;
-            GatherOut o{};
-            GatherCoef<T> c{};
-            o.grid = g;
-            o.local = h->sys.moms[j].local;
-            o.cls = h->comp_class[j];
-            o.src = h->src_slot[j];
-            for (int k = 0; k < n; ++k) {
-                double mx = h->sys.Mx[(size_t)j * n + k];
-                double my = h->sys.My[(size_t)j * n + k];
-                if (mx != 0.0) {
-                    if (h->sys.moms[k].grid != (g ^ 1) || o.nxt >= MAXC)
-                        return fail(h, STARMAP_E_UNSUPPORTED, "x-coupling outside the staggered pattern");
-                    o.xin[o.nxt] = h->sys.moms[k].local;
-                    c.cx[o.nxt] = (T)(-mx / h->dx);
-                    ++o.nxt;
-                }
-                if (my != 0.0) {
-                    if (h->sys.moms[k].grid != (g ^ 2) || o.nyt >= MAXC)
-                        return fail(h, STARMAP_E_UNSUPPORTED, "y-coupling outside the staggered pattern");
-                    o.yin[o.nyt] = h->sys.moms[k].local;
-                    c.cy[o.nyt] = (T)(-my / h->dy);
-                    ++o.nyt;
-                }
-            }
-            outs.push_back(o);
-            coefs.push_back(c);
-        }
-        h->tend[g] = (int)outs.size();
-    }
-    if (h->outs_dev) { cudaFree(h->outs_dev); h->outs_dev = nullptr; }
-    if (h->coefs_dev) { cudaFree(h->coefs_dev); h->coefs_dev = nullptr; }
-    CK(dev_alloc(&h->outs_dev, std::max<size_t>(1, outs.size()) * sizeof(GatherOut)), "cudaMalloc tables");
-    CK(dev_alloc(&h->coefs_dev, std::max<size_t>(1, coefs.size()) * sizeof(GatherCoef<T>)), "cudaMalloc tables");
-    if (!outs.empty()) {
-        CK(cudaMemcpy(h->outs_dev, outs.data(), outs.size() * sizeof(GatherOut), cudaMemcpyHostToDevice), "upload tables");
-        CK(cudaMemcpy(h->coefs_dev, coefs.data(), coefs.size() * sizeof(GatherCoef<T>), cudaMemcpyHostToDevice), "upload tables");
-    }
-    // source pointer array
-    std::vector<void*> ptrs(h->src_dev.begin(), h->src_dev.end());
-    if (h->src_ptrs_dev) { cudaFree(h->src_ptrs_dev); h->src_ptrs_dev = nullptr; }
-    CK(dev_alloc(&h->src_ptrs_dev, std::max<size_t>(1, ptrs.size()) * sizeof(void*)), "cudaMalloc sources");
-    if (!ptrs.empty())
-        CK(cudaMemcpy(h->src_ptrs_dev, ptrs.data(), ptrs.size() * sizeof(void*), cudaMemcpyHostToDevice), "upload sources");
     if (h->tiled) {
         int rc = tiled_update(h->tiled, h->sys, h->comp_class, h->src_slot, h->src_dev, h->frozen, h->dx, h->dy);
         if (rc) return fail(h, rc, tiled_error(h->tiled));
+        ++h->version;
+        return STARMAP_OK;
     }
-    if (!h->fp32 && h->cfg.system == STARMAP_PN2D) {
-        stream_destroy(h->stream64);
-        h->stream64 = nullptr;
-        if (stream_build(h->sys, h->comp_class, h->src_slot, h->frozen, h->dx, h->dy, &h->stream64))
-            return fail(h, STARMAP_E_CUDA, "cudaMalloc tables");
+    // source pointers by slot, at most one per component
+    std::vector<void*> ptrs(h->src_dev.begin(), h->src_dev.end());
+    ptrs.resize(h->ncomp, nullptr);
+    CK(table_upload(h->src_ptrs_dev, ptrs.data(), ptrs.size() * sizeof(void*)), "cudaMalloc sources");
+    if (!h->fp32 && h->cfg.system == STARMAP_PN2D && !h->stream64 && !h->stream_tried) {
+        if (stream_build(h->sys, h->frozen, h->dx, h->dy, &h->stream64))
+            return fail(h, STARMAP_E_CUDA, "streamed tables");
+        h->stream_tried = true;
+    }
+    if (h->stream64) {
+        if (stream_update(h->stream64, h->comp_class, h->src_slot)) return fail(h, STARMAP_E_CUDA, "cudaMalloc tables");
+    } else {
+        int rc = build_gather<T>(h);
+        if (rc) return rc;
     }
     ++h->version;
     return STARMAP_OK;
@@ -341,7 +357,7 @@ int run_pass(starmap_t* h, bool odd, int which) {
         a.p[1] = h->p[1];
         a.P = odd ? 1 : 0;
         a.which = which;
-        a.src = (double* const*)h->src_ptrs_dev;
+        a.src = (double* const*)h->src_ptrs_dev.p;
         if (stream_pass(h->stream64, a, h->stream)) return cuda_fail(h, cudaGetLastError(), "FP64 pass");
         return STARMAP_OK;
     }
@@ -360,9 +376,9 @@ int run_pass(starmap_t* h, bool odd, int which) {
     a.p[0] = h->p[0];
     a.p[1] = h->p[1];
     a.which = which;
-    a.outs = h->outs_dev;
-    a.coefs = (const GatherCoef<T>*)h->coefs_dev;
-    a.src = (T* const*)h->src_ptrs_dev;
+    a.outs = (const GatherOut*)h->outs_dev.p;
+    a.coefs = (const GatherCoef<T>*)h->coefs_dev.p;
+    a.src = (T* const*)h->src_ptrs_dev.p;
     if (launch_gather_pass<T>(a, h->stream)) return cuda_fail(h, cudaGetLastError(), "gather pass");
     return STARMAP_OK;
 }
@@ -557,9 +573,9 @@ void release(starmap_t* h) {
         if (h->prev[g]) cudaFree(h->prev[g]);
     }
     for (void* p : h->src_dev) if (p) cudaFree(p);
-    if (h->src_ptrs_dev) cudaFree(h->src_ptrs_dev);
-    if (h->outs_dev) cudaFree(h->outs_dev);
-    if (h->coefs_dev) cudaFree(h->coefs_dev);
+    table_free(h->src_ptrs_dev);
+    table_free(h->outs_dev);
+    table_free(h->coefs_dev);
     if (h->partials) cudaFree(h->partials);
     if (h->result) cudaFree(h->result);
     if (h->net_params) cudaFree(h->net_params);

@@ -42,6 +42,31 @@ inline cudaError_t dev_alloc(T** p, size_t bytes) {
     return cudaMalloc(reinterpret_cast<void**>(p), bytes);
 }
 
+// A table on the device: one allocation, kept while what is uploaded fits it
+// (a handle's tables keep their sizes when a source or a material changes).
+// Only with nothing in flight that reads it; it has landed on return.
+struct DevTable {
+    void* p = nullptr;
+    size_t cap = 0;
+};
+inline void table_free(DevTable& t) {
+    if (t.p) cudaFree(t.p);
+    t = DevTable();
+}
+inline cudaError_t table_upload(DevTable& t, const void* src, size_t bytes) {
+    if (!t.p || bytes > t.cap) {
+        table_free(t);
+        const size_t cap = bytes > 0 ? bytes : 1;
+        const cudaError_t e = dev_alloc(&t.p, cap);
+        if (e != cudaSuccess) return e;
+        t.cap = cap;
+    }
+    if (bytes == 0) return cudaSuccess;
+    const cudaError_t e = cudaMemcpy(t.p, src, bytes, cudaMemcpyHostToDevice);
+    // (a copy from pageable memory may return before its last part has landed)
+    return e == cudaSuccess ? cudaStreamSynchronize(cudaStreamLegacy) : e;
+}
+
 constexpr int LEAD = 32;          // elements before base_g
 constexpr int MAXC = 4;           // couplings per direction per row (Lemma 2)
 

@@ -24,17 +24,26 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 
 #include "pdl.h"
 #include "stream.h"
 
 namespace starmap {
 
+// The records of one pass and kind, with the component each of them completes
+// (-1: none).
+struct Records {
+    std::vector<StreamRec> rec;
+    std::vector<PairRec> pair;
+    std::vector<int> rec_comp, pair_comp;
+    size_t rec_at = 0, pair_at = 0;                                    // bytes into the device buffer
+};
+
 struct StreamTables {
-    StreamRec* rec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};   // [P][K]
-    PairRec* pair[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};    // [P][K]
-    int count[2] = {0, 0};                                             // stages of pass P
-    int outs[2][2] = {{0, 0}, {0, 0}};                                 // outputs of pass P, kind K
+    Records r[2][2];                                                   // [P][K]
+    std::vector<unsigned char> image;                                  // of the device buffer
+    DevTable dev;
     int slots = 0;                                                     // partial sums per thread
     double rho = 1.0;                                                  // dx / dy
     int sms = 1;
@@ -283,9 +292,8 @@ int comp_index(int l, int m, int imag) { return l * (l + 1) / 2 + (m > 0 ? 2 * (
 int nq(int l) { return l < 0 ? 0 : l / 2 + 1; }
 
 // Records of pass P and kind K; false where the system lacks the structure.
-bool build_records(const SystemMatrices& sys, const std::vector<int>& comp_class, const std::vector<int>& src_slot,
-                   const std::vector<char>& frozen, int P, int K, double dx, double dy, std::vector<StreamRec>& out,
-                   std::vector<PairRec>& pairs) {
+bool build_records(const SystemMatrices& sys, const std::vector<char>& frozen, int P, int K, double dx, double dy,
+                   Records& R) {
     const int n = sys.ncomp;
     const int N = sys.moms[n - 1].l;
     const int gin[2] = {P == 1 ? 0 : 1, P == 1 ? 3 : 2}, gout[2] = {P == 1 ? 1 : 0, P == 1 ? 2 : 3};
@@ -311,12 +319,15 @@ bool build_records(const SystemMatrices& sys, const std::vector<int>& comp_class
     };
     const double r = K == 0 ? -1.0 : 1.0;       // Pm and N0; the opposite for P0 and Np
     const int first = 1 - P;
-    auto finish = [&](StreamRec& e, int L, int q) {
+    auto finish = [&](StreamRec& e, int L, int q) -> int {
         const int j = comp(L, q, K);
-        if (j < 0 || frozen[j]) return;
+        if (j < 0 || frozen[j]) return -1;
         e.out = (int16_t)sys.moms[j].local;
-        e.cls = (int8_t)comp_class[j];
-        e.src = (int16_t)src_slot[j];
+        return j;
+    };
+    auto add = [&](const StreamRec& e, int j) {
+        R.rec.push_back(e);
+        R.rec_comp.push_back(j);
     };
     const StreamRec none = {0.0, 0.0, 0.0, 0.0, -1, -1, -1, -1, 0, -1, -1, -1, OP_NONE, {0, 0, 0}};
     int last = first;
@@ -325,10 +336,11 @@ bool build_records(const SystemMatrices& sys, const std::vector<int>& comp_class
         const int nin = nq(lp), nqp = lp > first ? nq(lp - 1) : 0;
         for (int q = 0; q < nin + (lp & 1); ++q) {
             StreamRec e = none;
+            int target = -1;
             if (q > 0) {
                 e.p0 = weight(lp - 1, q - 1, lp, q - 1, -r);
                 e.np = weight(lp + 1, q, lp, q - 1, -r);
-                finish(e, lp - 1, q - 1);
+                target = finish(e, lp - 1, q - 1);
             }
             if (q < nin) {
                 const int own = comp(lp, q, K), other = comp(lp, q, 1 - K);
@@ -350,15 +362,15 @@ bool build_records(const SystemMatrices& sys, const std::vector<int>& comp_class
             if (q < nin && none_in) ok = false;
             if (q < nin && later && !both) ok = false;
             if (lp + 1 <= N && q < nq(lp + 1)) e.store = (int8_t)q;
-            out.push_back(e);
+            add(e, target);
         }
     }
     if (last + 1 <= N)
         for (int q = 0; q < nq(last + 1); ++q) {
             StreamRec e = none;
             e.pre = (int8_t)q;
-            finish(e, last + 1, q);
-            out.push_back(e);
+            const int target = finish(e, last + 1, q);
+            add(e, target);
         }
     // the same sums output by output
     for (int j = 0; j < n; ++j) {
@@ -380,9 +392,8 @@ bool build_records(const SystemMatrices& sys, const std::vector<int>& comp_class
             covered = had;
         }
         p.out = (int16_t)m.local;
-        p.src = (int16_t)src_slot[j];
-        p.cls = (int8_t)comp_class[j];
-        pairs.push_back(p);
+        R.pair.push_back(p);
+        R.pair_comp.push_back(j);
     }
     // every target of the kind once, every coupling once
     long targets = 0, total = 0;
@@ -392,55 +403,69 @@ bool build_records(const SystemMatrices& sys, const std::vector<int>& comp_class
         for (int k = 0; k < n; ++k)
             total += (sys.Mx[(size_t)j * n + k] != 0.0) + (sys.My[(size_t)j * n + k] != 0.0);
     }
-    for (const StreamRec& e : out) targets -= e.out >= 0;
+    for (const StreamRec& e : R.rec) targets -= e.out >= 0;
     return ok && targets == 0 && covered == total;
 }
 
 }  // namespace
 
-int stream_build(const SystemMatrices& sys, const std::vector<int>& comp_class, const std::vector<int>& src_slot,
-                 const std::vector<char>& frozen, double dx, double dy, StreamTables** out) {
+int stream_build(const SystemMatrices& sys, const std::vector<char>& frozen, double dx, double dy, StreamTables** out) {
     *out = nullptr;
-    std::vector<StreamRec> rec[2][2];
-    std::vector<PairRec> pair[2][2];
+    StreamTables* t = new StreamTables();
     for (int P = 0; P < 2; ++P)
         for (int K = 0; K < 2; ++K)
-            if (!build_records(sys, comp_class, src_slot, frozen, P, K, dx, dy, rec[P][K], pair[P][K])) return 0;
-    StreamTables* t = new StreamTables();
+            if (!build_records(sys, frozen, P, K, dx, dy, t->r[P][K])) {
+                delete t;
+                return 0;
+            }
     t->slots = nq(sys.moms[sys.ncomp - 1].l);
     t->rho = dx / dy;
+    size_t bytes = 0;
+    auto place = [&](size_t n) {
+        const size_t at = bytes;
+        bytes = (bytes + n + 255) / 256 * 256;
+        return at;
+    };
+    for (int P = 0; P < 2; ++P)
+        for (int K = 0; K < 2; ++K) {
+            Records& R = t->r[P][K];
+            R.rec_at = place(R.rec.size() * sizeof(StreamRec));
+            R.pair_at = place(R.pair.size() * sizeof(PairRec));
+        }
+    t->image.assign(bytes, 0);
     int dev = 0, most = 0;
     cudaGetDevice(&dev);
-    bool ok = cudaDeviceGetAttribute(&t->sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-              cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
-              cudaFuncSetAttribute(k_stream_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, most) == cudaSuccess;
-    for (int P = 0; P < 2; ++P) {
-        t->count[P] = (int)rec[P][0].size();
-        for (int K = 0; K < 2 && ok; ++K) {
-            const size_t bytes = rec[P][K].size() * sizeof(StreamRec);
-            ok = dev_alloc(&t->rec[P][K], std::max<size_t>(1, bytes)) == cudaSuccess &&
-                 cudaMemcpy(t->rec[P][K], rec[P][K].data(), bytes, cudaMemcpyHostToDevice) == cudaSuccess;
-            t->outs[P][K] = (int)pair[P][K].size();
-            const size_t pb = pair[P][K].size() * sizeof(PairRec);
-            ok = ok && dev_alloc(&t->pair[P][K], std::max<size_t>(1, pb)) == cudaSuccess &&
-                 (pb == 0 || cudaMemcpy(t->pair[P][K], pair[P][K].data(), pb, cudaMemcpyHostToDevice) == cudaSuccess);
-        }
-    }
-    if (!ok) {
-        stream_destroy(t);
+    if (cudaDeviceGetAttribute(&t->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+        cudaFuncSetAttribute(k_stream_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess) {
+        delete t;
         return -4;
     }
     *out = t;
     return 0;
 }
 
-void stream_destroy(StreamTables* t) {
-    if (!t) return;
+int stream_update(StreamTables* t, const std::vector<int>& comp_class, const std::vector<int>& src_slot) {
     for (int P = 0; P < 2; ++P)
         for (int K = 0; K < 2; ++K) {
-            if (t->rec[P][K]) cudaFree(t->rec[P][K]);
-            if (t->pair[P][K]) cudaFree(t->pair[P][K]);
+            Records& R = t->r[P][K];
+            auto set = [&](auto& e, int j) {
+                if (j < 0) return;
+                e.cls = (int8_t)comp_class[j];
+                e.src = (int16_t)src_slot[j];
+            };
+            for (size_t i = 0; i < R.rec.size(); ++i) set(R.rec[i], R.rec_comp[i]);
+            for (size_t i = 0; i < R.pair.size(); ++i) set(R.pair[i], R.pair_comp[i]);
+            std::memcpy(t->image.data() + R.rec_at, R.rec.data(), R.rec.size() * sizeof(StreamRec));
+            if (!R.pair.empty())
+                std::memcpy(t->image.data() + R.pair_at, R.pair.data(), R.pair.size() * sizeof(PairRec));
         }
+    return table_upload(t->dev, t->image.data(), t->image.size()) == cudaSuccess ? 0 : -4;
+}
+
+void stream_destroy(StreamTables* t) {
+    if (!t) return;
+    table_free(t->dev);
     delete t;
 }
 
@@ -454,13 +479,15 @@ int stream_pass(const StreamTables* t, const StreamArgs& a, void* stream) {
         k.other[K] = a.g[gin[1 - K]];
         k.out[K] = a.g[gout[K]];
         k.out_grid[K] = gout[K];
-        k.rec[K] = t->rec[P][K];
-        k.pair[K] = t->pair[P][K];
-        k.outs[K] = t->outs[P][K];
+        const Records& R = t->r[P][K];
+        const unsigned char* dev = static_cast<const unsigned char*>(t->dev.p);
+        k.rec[K] = reinterpret_cast<const StreamRec*>(dev + R.rec_at);
+        k.pair[K] = reinterpret_cast<const PairRec*>(dev + R.pair_at);
+        k.outs[K] = (int)R.pair.size();
         k.slices[K] = 0;
         points = std::max(points, (long)k.out[K].nx * k.out[K].ny);
     }
-    k.count = t->count[P];
+    k.count = (int)t->r[P][0].rec.size();
     k.slots = t->slots;
     k.which = a.which;
     k.pitch = a.pitch;

@@ -54,10 +54,12 @@ struct StreamArgs {
     double* const* src;     // source arrays [ny][cp] by slot
 };
 
-// Tables of both passes; null (and nothing allocated) where the order's
-// couplings do not have the structure the kernel streams.  Returns 0 or -4.
-int stream_build(const SystemMatrices& sys, const std::vector<int>& comp_class, const std::vector<int>& src_slot,
-                 const std::vector<char>& frozen, double dx, double dy, StreamTables** out);
+// Tables of both passes, on the host; null where the order's couplings do not
+// have the structure the kernel streams.  Returns 0 or -4.
+int stream_build(const SystemMatrices& sys, const std::vector<char>& frozen, double dx, double dy, StreamTables** out);
+// Decay classes and source slots of the components; uploads the tables, into
+// one buffer that the first call allocates.  Returns 0 or -4.
+int stream_update(StreamTables* t, const std::vector<int>& comp_class, const std::vector<int>& src_slot);
 void stream_destroy(StreamTables* t);
 int stream_pass(const StreamTables* t, const StreamArgs& a, void* stream);
 

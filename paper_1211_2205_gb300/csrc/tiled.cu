@@ -142,12 +142,13 @@ struct TiledPlan {
     int* err_dev = nullptr;
     CUtensorMap maps_in[4], maps_out[4];
     PassTables tab[2];
-    void* dev_stages[2] = {nullptr, nullptr};
-    void* dev_rec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};    // [P][K]
-    // the fused step's tables
+    DevTable dev_stages[2];
+    DevTable dev_rec[2][2];               // [P][K]
+    // the fused step's tables (on the device only where there is one)
     int nin[2] = {0, 0}, nfin[2] = {0, 0};
-    void* dev_coef[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};   // [P][K]
-    void* dev_fin[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
+    std::vector<float> coef_rows[2][2];   // [P][K]
+    std::vector<int4> fin_rows[2][2];
+    DevTable dev_coef[2][2], dev_fin[2][2];
     int tiles_x = 0, tiles_y = 0;
     int variant = 0;                      // 0: 10-row tiles, 1: 5-row tiles
     int shape = 0;                        // index into kVariant
@@ -161,7 +162,7 @@ struct TiledPlan {
     bool fused = false;
     void* base1[4] = {nullptr, nullptr, nullptr, nullptr};   // the second buffer set
     fused::FusedParams fprm[2];           // [dir]: 0 set 0 -> set 1, 1 set 1 -> set 0
-    void* dev_odep = nullptr;
+    DevTable dev_odep;
     int fsmem = 0;
     int ftiles_x = 0, ftiles_y = 0;
     bool fready = false;
@@ -171,26 +172,19 @@ namespace {
 
 void free_tables(TiledPlan* pl) {
     for (int P = 0; P < 2; ++P) {
-        if (pl->dev_stages[P]) cudaFree(pl->dev_stages[P]);
-        pl->dev_stages[P] = nullptr;
+        table_free(pl->dev_stages[P]);
         for (int K = 0; K < 2; ++K) {
-            if (pl->dev_coef[P][K]) cudaFree(pl->dev_coef[P][K]);
-            if (pl->dev_fin[P][K]) cudaFree(pl->dev_fin[P][K]);
-            if (pl->dev_rec[P][K]) cudaFree(pl->dev_rec[P][K]);
-            pl->dev_coef[P][K] = pl->dev_fin[P][K] = pl->dev_rec[P][K] = nullptr;
+            table_free(pl->dev_coef[P][K]);
+            table_free(pl->dev_fin[P][K]);
+            table_free(pl->dev_rec[P][K]);
         }
     }
-    if (pl->dev_odep) cudaFree(pl->dev_odep);
-    pl->dev_odep = nullptr;
-    pl->fready = false;
+    table_free(pl->dev_odep);
 }
 
 template <class V>
-bool upload(void** dst, const std::vector<V>& v) {
-    size_t bytes = std::max<size_t>(1, v.size()) * sizeof(V);
-    if (dev_alloc(dst, bytes) != cudaSuccess) return false;
-    if (!v.empty() && cudaMemcpy(*dst, v.data(), v.size() * sizeof(V), cudaMemcpyHostToDevice) != cudaSuccess) return false;
-    return true;
+bool upload(DevTable& t, const std::vector<V>& v) {
+    return table_upload(t, v.data(), v.size() * sizeof(V)) == cudaSuccess;
 }
 
 // Walk the consumer loop of pass P and emit its tables.
@@ -340,9 +334,11 @@ int build_fused(TiledPlan* pl) {
         }
         odep[k] = run;
     }
-    if (pl->dev_odep) cudaFree(pl->dev_odep);
-    pl->dev_odep = nullptr;
-    if (!upload(&pl->dev_odep, odep)) { pl->err = "uploading the fused tables failed"; return -4; }
+    bool up = upload(pl->dev_odep, odep);
+    for (int P = 0; P < 2; ++P)
+        for (int K = 0; K < 2; ++K)
+            up = up && upload(pl->dev_coef[P][K], pl->coef_rows[P][K]) && upload(pl->dev_fin[P][K], pl->fin_rows[P][K]);
+    if (!up) { pl->err = "uploading the fused tables failed"; return -4; }
     // shared memory: barriers, two rings, both machines' tables, odep, partial sums
     auto al16 = [](int v) { return (v + 15) & ~15; };
     int tab = 0;
@@ -414,8 +410,8 @@ int build_fused(TiledPlan* pl) {
                 m.out[k].nx = pl->geo.nx[g];
                 m.out[k].ny = pl->geo.ny[g];
                 m.out[k].cp = pl->geo.cp[g];
-                m.coef[k] = (const float4*)pl->dev_coef[P][k];
-                m.fin[k] = (const int4*)pl->dev_fin[P][k];
+                m.coef[k] = (const float4*)pl->dev_coef[P][k].p;
+                m.fin[k] = (const int4*)pl->dev_fin[P][k].p;
                 m.smem_coef_off[k] = tables + coef_rel[M][k];
                 m.smem_fin_off[k] = tables + fin_rel[M][k];
             }
@@ -428,7 +424,7 @@ int build_fused(TiledPlan* pl) {
             m.smem_part_off = tables + part_rel[M];
             m.ring_off = M == 0 ? ering : oring;
         }
-        fp.odep = (const int*)pl->dev_odep;
+        fp.odep = (const int*)pl->dev_odep.p;
         fp.smem_odep_off = tables + odep_rel;
         fp.pitch = pitch;
         fp.p[0] = pl->geo.p[0];
@@ -506,8 +502,7 @@ int tiled_create(const TiledGeometry& geo, TiledPlan** out) {
 int tiled_update(TiledPlan* pl, const SystemMatrices& sys, const std::vector<int>& comp_class,
                  const std::vector<int>& src_slot, const std::vector<void*>& src_dev,
                  const std::vector<char>& frozen, double dx, double dy) {
-    free_tables(pl);
-    pl->ready = false;
+    pl->ready = pl->fready = false;
     if (pl->variant == 0 && pl->N > TALL_TILE_MAX_N) {
         pl->err = "tiled kernel needs more shared memory than the device offers";
         return -8;
@@ -521,9 +516,9 @@ int tiled_update(TiledPlan* pl, const SystemMatrices& sys, const std::vector<int
         // y part of the other input) and finalise entries (offset, source address)
         // (each value once: the kernel pairs it for f32x2 itself)
         const size_t nsteps = t.coef.size() / 32;
-        std::vector<float> ck[2];
+        std::vector<float>(&ck)[2] = pl->coef_rows[P];
         for (int K = 0; K < 2; ++K) {
-            ck[K].resize(nsteps * 8);
+            ck[K].assign(nsteps * 8, 0.f);
             for (size_t k = 0; k < nsteps; ++k) {
                 const float* rowK = t.coef.data() + 32 * k + 16 * K;
                 const float* rowO = t.coef.data() + 32 * k + 16 * (1 - K);
@@ -533,7 +528,8 @@ int tiled_update(TiledPlan* pl, const SystemMatrices& sys, const std::vector<int
                 }
             }
         }
-        std::vector<int4> fk[2];
+        std::vector<int4>(&fk)[2] = pl->fin_rows[P];
+        for (int K = 0; K < 2; ++K) fk[K].clear();
         for (size_t e = 0; e + 1 < t.fin.size() + 1; e += 2) {
             for (int K = 0; K < 2; ++K) {
                 const int comp = t.fin_comp[e + K];
@@ -550,18 +546,13 @@ int tiled_update(TiledPlan* pl, const SystemMatrices& sys, const std::vector<int
                 fk[K].push_back(make_int4((int)(off / 32), 0, (int)(unsigned)src, (int)(unsigned)(src >> 32)));
             }
         }
-        for (int K = 0; K < 2; ++K)
-            if (!upload(&pl->dev_coef[P][K], ck[K]) || !upload(&pl->dev_fin[P][K], fk[K])) {
-                pl->err = "uploading the tiled tables failed";
-                return -4;
-            }
         pl->nin[P] = (int)nsteps;
         pl->nfin[P] = (int)fk[0].size();
         // an absent I input is loaded as a box of zeros: a component outside the tensor
         std::vector<int4> st = t.stages;
         for (int4& v : st)
             if (v.x >= 0 && v.y < 0) v.y = std::max(1, pl->geo.K[gin[P][1]]);
-        if (!upload(&pl->dev_stages[P], st)) {
+        if (!upload(pl->dev_stages[P], st)) {
             pl->err = "uploading the tiled tables failed";
             return -4;
         }
@@ -592,7 +583,7 @@ int tiled_update(TiledPlan* pl, const SystemMatrices& sys, const std::vector<int
                 in += has_in;
             }
             if (in != nsteps || fin != fk[K].size()) { pl->err = "tiled stage list and tables differ"; return -8; }
-            if (!upload(&pl->dev_rec[P][K], rk[K])) { pl->err = "uploading the tiled tables failed"; return -4; }
+            if (!upload(pl->dev_rec[P][K], rk[K])) { pl->err = "uploading the tiled tables failed"; return -4; }
         }
         // shared memory: barriers, partial sums, records, stages, ring.  The
         // ring takes what the resident CTAs leave
@@ -657,9 +648,9 @@ int tiled_update(TiledPlan* pl, const SystemMatrices& sys, const std::vector<int
             prm.nstages = (int)t.stages.size();
             prm.nring = nring;
             prm.top = t.top;
-            prm.stages = (const int4*)pl->dev_stages[P];
+            prm.stages = (const int4*)pl->dev_stages[P].p;
             for (int K = 0; K < 2; ++K) {
-                prm.rec[K] = (const float4*)pl->dev_rec[P][K];
+                prm.rec[K] = (const float4*)pl->dev_rec[P][K].p;
                 prm.smem_rec_off[K] = rec_off[K];
             }
             prm.err = pl->err_dev;
