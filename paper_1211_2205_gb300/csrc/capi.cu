@@ -7,6 +7,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -267,6 +268,34 @@ int build_tables(starmap_t* h) {
 
 int rebuild_tables(starmap_t* h) {
     return h->fp32 ? build_tables<float>(h) : build_tables<double>(h);
+}
+
+// Rows of nx values to device rows of cp.  A 2D copy of pageable memory takes
+// 5 to 7 us longer than a plain one (replacing a source, FP64 and FP32 64^2:
+// 18.8 and 11.5 us, FP32 150^2: 38 and 33), so the copy is plain where it
+// needs no further pass over the values: rows without padding, and FP32, whose
+// conversion writes padded rows as well.  (FP64 padded on the host: 100^2 24 ->
+// 27 us, 1023 x 700 514 -> 863; a narrow FP32 grid would mostly send padding.)
+template <class T>
+cudaError_t upload_rows(void* d, const double* q, int nx, int ny, int cp) {
+    const size_t row = (size_t)nx * sizeof(T), pitch = (size_t)cp * sizeof(T);
+    const bool convert = sizeof(T) != sizeof(double);
+    std::unique_ptr<T[]> rows;
+    const void* from = q;
+    int w = nx;                                         // of a row at `from`
+    if (convert) {
+        if (cp <= 2 * nx) w = cp;
+        rows.reset(new T[(size_t)w * ny]);
+        if (w == nx) std::copy(q, q + (size_t)nx * ny, rows.get());
+        else
+            for (int y = 0; y < ny; ++y) {
+                T* r = std::copy(q + (size_t)y * nx, q + (size_t)(y + 1) * nx, rows.get() + (size_t)y * w);
+                std::fill(r, rows.get() + (size_t)(y + 1) * w, T(0));
+            }
+        from = rows.get();
+    }
+    return w == cp ? cudaMemcpy(d, from, pitch * ny, cudaMemcpyHostToDevice)
+                   : cudaMemcpy2D(d, pitch, from, row, row, ny, cudaMemcpyHostToDevice);
 }
 
 // Decay coefficients of grid g from the stored material (section 5.5/5.7):
@@ -1008,11 +1037,8 @@ int starmap_set_source(starmap_t* h, int j, const double* q, size_t count) {
     double sq = 0.0;
     for (size_t i = 0; i < np; ++i) sq += q[i] * q[i];
     h->src_sq[j] = sq;
-    std::vector<float> tmp;
-    if (h->fp32) tmp.assign(q, q + np);
-    const size_t row = h->nxg[g] * h->esize;
-    CK(cudaMemcpy2D(d, h->cpg[g] * h->esize, h->fp32 ? (const void*)tmp.data() : (const void*)q, row, row, h->nyg[g],
-                    cudaMemcpyHostToDevice), "upload source");
+    const int nx = h->nxg[g], ny = h->nyg[g], cp = h->cpg[g];
+    CK(h->fp32 ? upload_rows<float>(d, q, nx, ny, cp) : upload_rows<double>(d, q, nx, ny, cp), "upload source");
     // the pass tables only change when a component gains a source
     return new_slot ? rebuild_tables(h) : STARMAP_OK;
 }
