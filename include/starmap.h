@@ -570,9 +570,9 @@ int  starmap_batch_tile_rows(const starmap_batch_t* b, double* ms_tall, double* 
  * from timing (0).  The autotuner (kernel AUTO) builds the batch with each
  * tile height, plans its work units with each strip length, times four
  * steps of every candidate and keeps the fastest; it caches the choice in a
- * text file keyed by the device and every instance's system, order, cells,
- * boundaries and schedule, so a later batch of the same shapes skips the
- * timing.  The file is $STARMAP_TUNE_CACHE, else
+ * text file keyed by the batch kernel's sources, the device and every
+ * instance's system, order, cells, boundaries and schedule, so a later batch
+ * of the same shapes on the same build skips the timing.  The file is $STARMAP_TUNE_CACHE, else
  * $HOME/.cache/starmap/batch_tune.txt; STARMAP_TUNE_CACHE=off disables it.
  * A file that cannot be read or written only means no cache. */
 int  starmap_batch_tuning(const starmap_batch_t* b, int* tile_rows, int* strip_stages, int* from_cache);

@@ -8,6 +8,7 @@ without a GPU driver (the symbol-export tests run there).
 from __future__ import annotations
 
 import concurrent.futures
+import hashlib
 import os
 import shutil
 import subprocess
@@ -27,6 +28,9 @@ CXX_FLAGS = ["-O2", "-fPIC", "-std=c++17", "-I", CSRC]
 SOURCES = ["host_math.cpp", "kernels_gather.cu", "kernels_stream.cu", "tiled.cu", "capi.cu", "noalloc.cu", "mlp.cu", "mlp_tc.cu", "mlp_capi.cu"]
 HEADERS = ["host_math.h", "internal.h", "stream.h", "tiled.h", "tiled_kernel.cuh", "fused_kernel.cuh", "mlp.h", "closure_features.cuh",
            "pdl.h"]
+# What a batch's tuning was measured on: the kernel, its host side and the
+# planner.  Their hash is part of the tuning cache's key (capi.cu).
+BATCH_SOURCES = ["tiled_kernel.cuh", "pdl.h", "tiled.cu", "capi.cu"]
 
 
 def _nvcc() -> str:
@@ -36,8 +40,17 @@ def _nvcc() -> str:
     raise RuntimeError("nvcc not found")
 
 
-def _deps_mtime() -> float:
-    files = [os.path.join(CSRC, f) for f in HEADERS]
+def batch_sources_hash() -> str:
+    """First 16 hex digits of the SHA-256 of BATCH_SOURCES."""
+    h = hashlib.sha256()
+    for f in BATCH_SOURCES:
+        with open(os.path.join(CSRC, f), "rb") as fp:
+            h.update(fp.read())
+    return h.hexdigest()[:16]
+
+
+def _deps_mtime(src: str) -> float:
+    files = [os.path.join(CSRC, f) for f in HEADERS + (BATCH_SOURCES if src == "capi.cu" else [])]
     files.append(os.path.join(os.path.dirname(HERE), "include", "starmap.h"))
     return max(os.path.getmtime(f) for f in files if os.path.exists(f))
 
@@ -46,10 +59,12 @@ def _compile(src: str, extra: list, verbose: bool) -> str:
     path = os.path.join(CSRC, src)
     obj = os.path.join(BUILD, src + ".o")
     if (os.path.exists(obj) and os.path.getmtime(obj) >= os.path.getmtime(path)
-            and os.path.getmtime(obj) >= _deps_mtime()):
+            and os.path.getmtime(obj) >= _deps_mtime(src)):
         return obj
     if src.endswith(".cu"):
         cmd = [_nvcc(), "-c", path, "-o", obj] + NVCC_FLAGS + extra
+        if src == "capi.cu":
+            cmd.append(f'-DSTARMAP_BATCH_SOURCES="{batch_sources_hash()}"')
     else:
         cmd = [os.environ.get("CXX", "g++"), "-c", path, "-o", obj] + CXX_FLAGS + [
             "-I", "/usr/local/cuda/include"]

@@ -1859,14 +1859,21 @@ std::string tune_cache_path() {
     return home ? std::string(home) + "/.cache/starmap/batch_tune.txt" : std::string();
 }
 
-// FNV-1a over the device (name, SM count) and every instance's system,
-// order, cells, boundaries and schedule.
+// The build's hash of the sources a tuning depends on (build.py); compiled
+// without it, the time of compilation.
+#ifndef STARMAP_BATCH_SOURCES
+#define STARMAP_BATCH_SOURCES __DATE__ " " __TIME__
+#endif
+
+// FNV-1a over the batch kernel's sources, the device (name, SM count) and
+// every instance's system, order, cells, boundaries and schedule.
 std::string batch_signature(const starmap_config* cfgs, int count) {
     unsigned long long hsh = 1469598103934665603ull;
     auto mix = [&](const void* p, size_t n) {
         const unsigned char* c = static_cast<const unsigned char*>(p);
         for (size_t i = 0; i < n; ++i) { hsh ^= c[i]; hsh *= 1099511628211ull; }
     };
+    mix(STARMAP_BATCH_SOURCES, sizeof(STARMAP_BATCH_SOURCES));
     int dev = 0;
     cudaDeviceProp prop;
     if (cudaGetDevice(&dev) == cudaSuccess && cudaGetDeviceProperties(&prop, dev) == cudaSuccess) {

@@ -191,3 +191,27 @@ def test_autotuner_cache(tmp_path, monkeypatch):
     other = capi.Batch.from_problems(probs[:2])          # another signature: tuned again
     assert not other.tuning()[2]
     assert len(path.read_text().splitlines()) == 2
+
+
+def test_autotuner_cache_of_other_kernels(tmp_path, monkeypatch):
+    """A choice measured on other kernels is not taken: the file holds a line
+    keyed by the device and the shapes alone, as files of earlier builds do."""
+    import struct
+
+    import torch
+    path = tmp_path / "tune.txt"
+    monkeypatch.setenv("STARMAP_TUNE_CACHE", str(path))
+    probs = [_instance(k, nsteps=3) for k in range(3)]
+    dev = torch.cuda.get_device_properties(0)
+    bc = {"periodic": capi.PERIODIC, "extrapolation": capi.EXTRAPOLATION}
+    key = dev.name.encode() + struct.pack("ii", dev.multi_processor_count, len(probs))
+    for p in probs:
+        key += struct.pack("7i", capi.PN2D, p.N, *p.n, *[bc[b] for b in p.bc], capi.SCHEDULE_MERGED)
+    h = 1469598103934665603
+    for byte in key:
+        h = (h ^ byte) * 1099511628211 % (1 << 64)
+    path.write_text(f"{h:016x} 5 96 0.100000\n")
+    b = capi.Batch.from_problems(probs, schedule="merged")
+    assert not b.tuning()[2]
+    again = capi.Batch.from_problems(probs, schedule="merged")
+    assert again.tuning()[2]
