@@ -44,9 +44,11 @@ struct StreamTables {
     Records r[2][2];                                                   // [P][K]
     std::vector<unsigned char> image;                                  // of the device buffer
     DevTable dev;
+    int N = 1;
     int slots = 0;                                                     // partial sums per thread
     double rho = 1.0;                                                  // dx / dy
     int sms = 1;
+    int resident[2] = {1, 1};                                          // streaming blocks on an SM, pass P
 };
 
 namespace {
@@ -57,6 +59,8 @@ struct KernelArgs {
     const PairRec* pair[2];
     int outs[2], slices[2];     // k_pair_pass: outputs of a kind, blockIdx.y's slices of them
     int out_grid[2];
+    // slots is not read by the kernels: with these two others alone the compiler gives k_stream_pass 64 registers
+    // instead of 70, and P_63 takes 2 % longer, P_13 2 % at 256^2 (and 1 % less at 512^2)
     int count, slots, which;
     long pitch;
     int p[2];
@@ -139,7 +143,10 @@ __device__ __forceinline__ double pair_sum(const PairRec& r, const double (&v)[4
 // and coefficients, host-written, are loaded before the previous pass is
 // waited for.  100^2 P_5: 13 us per pass with a launch per grid, tables in
 // local memory and no overlap, 5.5 so.
-__global__ void __launch_bounds__(128) k_pair_pass(const __grid_constant__ KernelArgs A) {
+// Wide: the same on large grids of N <= 2, where the streamed chain is too
+// short to be worth its stages and the warps in flight are what counts: 64
+// registers instead of 94.
+__device__ __forceinline__ void pair_pass(const KernelArgs& A) {
     pdl_trigger();
     const int K = (int)blockIdx.y < A.slices[0] ? 0 : 1;
     const int slice = (int)blockIdx.y - (K ? A.slices[0] : 0);
@@ -184,11 +191,15 @@ __global__ void __launch_bounds__(128) k_pair_pass(const __grid_constant__ Kerne
     if (!waited) pdl_wait();
 }
 
+constexpr int THREADS = 128;
+__global__ void __launch_bounds__(THREADS) k_pair_pass(const __grid_constant__ KernelArgs A) { pair_pass(A); }
+__global__ void __launch_bounds__(THREADS, 8) k_pair_pass_wide(const __grid_constant__ KernelArgs A) { pair_pass(A); }
+
 // Seven blocks of 128 on an SM (up to N = 39 or so): a pass over 256^2 points
 // is one wave of blocks.  256^2 P_13: 114 us per pass with the gather kernel,
 // 75 so.  (-rho is an operand modifier of the multiply-add here; with a second
 // register for it the compiler schedules the loop worse, 85.)
-__global__ void __launch_bounds__(128, 7) k_stream_pass(const __grid_constant__ KernelArgs A) {
+__global__ void __launch_bounds__(THREADS, 7) k_stream_pass(const __grid_constant__ KernelArgs A) {
     extern __shared__ __align__(16) unsigned char raw[];
     StreamRec* rec = reinterpret_cast<StreamRec*>(raw);
     const int K = blockIdx.y;
@@ -407,6 +418,10 @@ bool build_records(const SystemMatrices& sys, const std::vector<char>& frozen, i
     return ok && targets == 0 && covered == total;
 }
 
+size_t stream_smem(const StreamTables& t, int P) {
+    return t.r[P][0].rec.size() * sizeof(StreamRec) + (size_t)t.slots * THREADS * sizeof(double);
+}
+
 }  // namespace
 
 int stream_build(const SystemMatrices& sys, const std::vector<char>& frozen, double dx, double dy, StreamTables** out) {
@@ -418,7 +433,8 @@ int stream_build(const SystemMatrices& sys, const std::vector<char>& frozen, dou
                 delete t;
                 return 0;
             }
-    t->slots = nq(sys.moms[sys.ncomp - 1].l);
+    t->N = sys.moms[sys.ncomp - 1].l;
+    t->slots = nq(t->N);
     t->rho = dx / dy;
     size_t bytes = 0;
     auto place = [&](size_t n) {
@@ -441,6 +457,12 @@ int stream_build(const SystemMatrices& sys, const std::vector<char>& frozen, dou
         delete t;
         return -4;
     }
+    for (int P = 0; P < 2; ++P)
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&t->resident[P], k_stream_pass, THREADS, stream_smem(*t, P)) !=
+            cudaSuccess) {
+            delete t;
+            return -4;
+        }
     *out = t;
     return 0;
 }
@@ -496,21 +518,33 @@ int stream_pass(const StreamTables* t, const StreamArgs& a, void* stream) {
     k.rho = t->rho;
     k.minus_rho = -t->rho;
     k.src = a.src;
-    const int threads = 128;
-    const unsigned blocks = (unsigned)((points + threads - 1) / threads);
+    const long blocks = (points + THREADS - 1) / THREADS;
     cudaError_t e;
-    if (points >= 200L * t->sms) {
-        // two threads per point, whose chains of stages need about three
-        // warps per scheduler of the GPU to hide one another.  us per pass,
-        // output by output / streamed: 128^2 P_5 7.5 / 8.8, P_13 28 / 32,
-        // P_39 223 / 262; 181^2 13.0 / 13.7, 59 / 57, 494 / 446; 256^2 19.9 /
-        // 17.0, 103 / 75, 880 / 585
-        const size_t smem = (size_t)k.count * sizeof(StreamRec) + (size_t)k.slots * threads * sizeof(double);
-        e = launch_pdl(k_stream_pass, dim3(blocks, 2), dim3(threads), smem, (cudaStream_t)stream, blocks <= 1024, k);
+    // Streamed: two threads per point, whose chains of stages need about two
+    // warps per scheduler of the GPU to hide one another (the fewer stages, the
+    // more).  us per pass, output by output / streamed: P_3 200^2 7.8 / 8.3,
+    // 220^2 8.8 / 8.4, 512^2 33 / 28; P_5 175^2 11.7 / 12.3, 190^2 13.3 / 12.3,
+    // 256^2 21 / 16; P_7 175^2 19.1 / 18.4, P_13 54 / 45, P_39 429 / 336; 256^2
+    // P_13 112 / 74, P_39 905 / 585.  At N <= 2 an input has too few targets:
+    // P_2 512^2 16.6 (wide) / 18.7, P_1 7.8 / 12.3.
+    const long from = t->N >= 7 ? 200 : t->N >= 5 ? 230 : 300;
+    if (t->N > 2 && points >= from * t->sms) {
+        // A pass overlaps the previous one's tail only where that one's blocks
+        // fill the SMs evenly: early blocks take whatever slots it leaves, and
+        // an SM then runs its full number of them while another has a few.
+        // 220^2 P_13 (five blocks per SM of seven) 75 us with, 55 without; 175^2
+        // P_39 496 and 336; 256^2 P_5 (6.7 of seven) 16.3 and 18.1.
+        const bool overlap = blocks <= 1024 && 2 * blocks > (long)t->sms * (t->resident[P] - 1);
+        e = launch_pdl(k_stream_pass, dim3((unsigned)blocks, 2), dim3(THREADS), stream_smem(*t, P), (cudaStream_t)stream,
+                       overlap, k);
     } else {
-        // one output per thread (up to 64 slices per kind)
+        // one output per thread (up to 64 slices per kind).  Wide, us per pass,
+        // without / with: P_1 256^2 3.6 / 4.0, 350^2 5.6 / 4.9, 512^2 9.1 / 7.8,
+        // 1500 x 1300 57 / 47; P_2 256^2 6.7 / 6.1, 512^2 18.5 / 16.6, 1500 x 1300 137 / 115
         for (int K = 0; K < 2; ++K) k.slices[K] = std::min(k.outs[K], 64);
-        e = launch_pdl(k_pair_pass, dim3(blocks, k.slices[0] + k.slices[1]), dim3(threads), 0, (cudaStream_t)stream, true, k);
+        const bool wide = t->N <= 2 && points >= (t->N == 1 ? 500 : 400) * (long)t->sms;
+        e = launch_pdl(wide ? k_pair_pass_wide : k_pair_pass, dim3((unsigned)blocks, k.slices[0] + k.slices[1]),
+                       dim3(THREADS), 0, (cudaStream_t)stream, true, k);
     }
     return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? 0 : -4;
 }

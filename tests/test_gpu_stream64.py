@@ -63,3 +63,36 @@ def test_both_give_the_same_values(N):
         out.append([s.moments(j) for j in range(s.ncomp)])
     for a, b in zip(*out):
         assert np.array_equal(np.tile(a, (1, 4)), b)
+
+
+@pytest.mark.parametrize("n", [(331, 333), (223, 251)])
+@pytest.mark.parametrize("N", [1, 2, 3, 5, 7])
+def test_around_the_sizes_of_the_rules(N, n):
+    """331 x 333 points: wide output by output (N <= 2) or streamed with the
+    passes overlapped; 223 x 251: output by output (N <= 2) or streamed pass
+    after pass."""
+    p = _random_problem(N, n, ("extrapolation", "periodic"), "fp64", 780 + N, 3)
+    s, got = gpu_run(p, schedule="merged")
+    o, ref = oracle_run(p, s)
+    assert_parity(got, ref, FP64_TOL, "fp64")
+
+
+@pytest.mark.parametrize("N", [1, 2, 3, 5])
+def test_every_kernel_gives_the_same_values(N):
+    """As test_both_give_the_same_values, at sizes on both sides of the low
+    orders' rules: a row of sixteen copies equals the single one bit for bit."""
+    out = []
+    for rep in (1, 16):
+        s = capi.Stepper(N=N, ax=(0.0, float(rep), 0.0, 1.0), n=(96 * rep, 96), precision="fp64", schedule="merged")
+        for g in range(4):
+            X, Y = s.grid_coords(g)
+            v = np.tile(1.0 + 0.5 * np.sin(2 * np.pi * X[:, :96]) * np.cos(2 * np.pi * Y[:, :96]), (1, rep))
+            s.set_material(g, 0.3 * v, v)
+        for j in range(s.ncomp):
+            X, Y = s.grid_coords(s.moment_info(j)["grid"])
+            s.set_moment(j, np.tile(np.exp(np.cos(2 * np.pi * X[:, :96] + j) + np.sin(2 * np.pi * Y[:, :96])), (1, rep)))
+        s.set_source(0, np.tile(np.cos(2 * np.pi * s.grid_coords(0)[0][:, :96]), (1, rep)))
+        s.step(5)
+        out.append([s.moments(j) for j in range(s.ncomp)])
+    for a, b in zip(*out):
+        assert np.array_equal(np.tile(a, (1, 16)), b)
