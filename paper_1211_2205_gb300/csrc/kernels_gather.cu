@@ -152,19 +152,33 @@ __device__ __forceinline__ T add_terms(T w, int n, const T (&c)[MAXC], const T (
 // operations (64 clocks each, one at a time per warp) are the pass: the
 // tables and decay coefficients, host-written, are loaded before the
 // previous pass is waited for (pdl.h).
-template <class T>
-__global__ void __launch_bounds__(128) k_gather_pass(const __grid_constant__ GatherArgs<T> A) {
+// ROWS: a row of blocks per row of points (blockIdx.y), for long rows: no
+// division, and with more warps in flight (72 registers instead of 88) and
+// all loads of an output together.  us per pass, without / with: FP32 P_1
+// 1500^2 50 / 39, P_3 142 / 106, P_39 256^2 352 / 241; slab of 60000 cells
+// FP64 P_63 38 / 31.
+template <class T, bool ROWS>
+__device__ __forceinline__ void gather_pass(const GatherArgs<T>& A) {
     pdl_trigger();
+    if (ROWS) pdl_wait();
     const int K = (int)blockIdx.z < A.slices[0] ? 0 : 1;
     const int slice = (int)blockIdx.z - (K ? A.slices[0] : 0);
     const GridDev<T>& G = A.out[K];
     const int nx = G.nx, ny = G.ny;
-    // points in rows one after the other: no lanes idle at a row's end (an FP64 operation costs a warp of
-    // four lanes what it costs a whole one)
-    const unsigned long long point = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool inside = point < (unsigned long long)nx * ny;
-    const int iy = point >> 32 ? (int)(point / nx) : (int)((unsigned)point / (unsigned)nx);
-    const int ix = (int)(point - (unsigned long long)iy * nx);
+    int ix, iy;
+    bool inside;
+    if (ROWS) {
+        ix = blockIdx.x * blockDim.x + threadIdx.x;
+        iy = blockIdx.y;
+        inside = ix < nx && iy < ny;
+    } else {
+        // points in rows one after the other: no lanes idle at a row's end (an FP64 operation costs a warp of
+        // four lanes what it costs a whole one)
+        const unsigned long long point = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+        inside = point < (unsigned long long)nx * ny;
+        iy = point >> 32 ? (int)(point / nx) : (int)((unsigned)point / (unsigned)nx);
+        ix = (int)(point - (unsigned long long)iy * nx);
+    }
     const bool xnode = (A.grid[K] & 1) != 0, ynode = (A.grid[K] & 2) != 0;
     const long pitch = A.pitch;
     // right / upper neighbour in the partner grid (eq. central_differences)
@@ -174,7 +188,7 @@ __global__ void __launch_bounds__(128) k_gather_pass(const __grid_constant__ Gat
     T* self = G.base + (long)(iy + 1) * pitch + ix;
     const long cidx = inside ? (long)iy * G.cp + ix : 0;
     const long plane = (long)G.cp * ny;
-    bool waited = false;
+    bool waited = ROWS;
     for (int t = A.begin[K] + slice; t < A.end[K]; t += A.slices[K]) {
         const GatherOut o = A.outs[t];
         const GatherCoef<T> c = A.coefs[t];
@@ -206,6 +220,14 @@ __global__ void __launch_bounds__(128) k_gather_pass(const __grid_constant__ Gat
         store_point(comp, pitch, ix, iy, nx, ny, xnode, ynode, A.p[0], A.p[1], v);
     }
     if (!waited) pdl_wait();
+}
+template <class T>
+__global__ void __launch_bounds__(128) k_gather_pass(const __grid_constant__ GatherArgs<T> A) {
+    gather_pass<T, false>(A);
+}
+template <class T>
+__global__ void __launch_bounds__(128, 7) k_gather_rows(const __grid_constant__ GatherArgs<T> A) {
+    gather_pass<T, true>(A);
 }
 
 // Refresh the boundary copies of components [kbegin, kend) of one grid.
@@ -349,8 +371,18 @@ int launch_gather_pass(GatherArgs<T> a, void* stream) {
         const long z = threads >= want ? 1 : (want * std::max(n, 0) / outs + threads - 1) / threads;
         a.slices[K] = n <= 0 ? 0 : (int)std::min<long>(std::min<long>(std::max<long>(z, 1), n), 64);
     }
-    const dim3 grid((unsigned)(threads / width), 1, a.slices[0] + a.slices[1]);
-    const cudaError_t e = launch_pdl(k_gather_pass<T>, grid, dim3(width), 0, (cudaStream_t)stream, threads < want, a);
+    // By rows where a sixteenth of the lanes at most is idle for it, from the size on where the loads' latency
+    // and not the launch's counts.  us per pass, without / with: FP32 256^2 P_1 (98 k values) 2.3 / 3.2, P_7 12.9 /
+    // 12.1, 512^2 P_1 (393 k) 5.5 / 5.6, P_2 9.3 / 8.8; slabs of 10000 cells, FP64 P_15 (80 k) 2.9 / 4.2, P_31 5.2 /
+    // 4.9, FP32 P_63 (320 k) 5.0 / 5.1; 120 x 90 (a fifteenth idle) P_60 99 / 102
+    const int nxmax = std::max(a.out[0].nx, a.out[1].nx), nymax = std::max(a.out[0].ny, a.out[1].ny);
+    const int per_row = (nxmax + width - 1) / width;
+    const bool rows = points * outs >= (sizeof(T) == 8 ? 150000 : 500000) && 16L * per_row * width <= 17L * nxmax &&
+                      nymax <= 65535;
+    const dim3 grid = rows ? dim3(per_row, nymax, a.slices[0] + a.slices[1])
+                           : dim3((unsigned)(threads / width), 1, a.slices[0] + a.slices[1]);
+    const cudaError_t e = launch_pdl(rows ? k_gather_rows<T> : k_gather_pass<T>, grid, dim3(width), 0,
+                                     (cudaStream_t)stream, threads < want, a);
     return status_of(e != cudaSuccess ? e : cudaGetLastError());
 }
 
