@@ -117,3 +117,75 @@ def test_sources_in_every_moment():
     for a, b in zip(got[0], got[1]):
         assert np.array_equal(a, b)
     assert_parity(got[0], [np.asarray(a, np.float64) for a in got[2]], FP32_TOL, "fp32")
+
+
+def _with_sources(N, n, kernel, schedule="merged", aniso=True, steps=2):
+    p = _random_problem(N, n, ("periodic", "extrapolation"), "fp32", 991 + N, steps, aniso=aniso)
+    s = capi.Stepper.from_problem(p, kernel=kernel, schedule=schedule)
+    for j in range(s.ncomp):
+        X, Y = s.grid_coords(s.moment_info(j)["grid"])
+        s.set_source(j, np.cos(0.7 * j + 3 * X) * np.exp(-Y) / (1 + j % 7))
+    s.step(steps)
+    return [s.moments(j) for j in range(s.ncomp)]
+
+
+# above half of L2 with its sources: the five-row bands (more tiles than SMs, N <= 15), the two-row bands
+# with each weight once (N >= 50) and, with isotropic scattering, twice
+WARMED = [(15, (353, 351), True), (15, (353, 351), False), (9, (601, 399), False), (50, (101, 93), True),
+          (55, (101, 93), False), (35, (161, 137), False)]
+
+
+@pytest.mark.parametrize("N,n,aniso", WARMED)
+def test_sources_in_every_moment_shapes(N, n, aniso):
+    """As test_sources_in_every_moment, for the tile shapes and decay classes
+    that it does not reach; ragged in x and y."""
+    from helpers import assert_parity
+    from test_gpu_parity import FP32_TOL
+    tall = _with_sources(N, n, "tiled_tall", aniso=aniso)
+    short = _with_sources(N, n, "tiled_short", aniso=aniso)
+    for a, b in zip(tall, short):
+        assert np.array_equal(a, b)
+    gather = _with_sources(N, n, "gather", aniso=aniso)
+    assert_parity(tall, [np.asarray(a, np.float64) for a in gather], FP32_TOL, "fp32")
+
+
+# kernel, N, cells, sources in every moment: two-row bands, the same with each weight once, 5-row tiles, and
+# the warming variants of the two-row and five-row bands
+REPEATED = [("tiled_tall", 16, (1001, 799), False), ("tiled_tall", 50, (330, 290), False),
+            ("tiled_short", 9, (1501, 1099), False), ("tiled_tall", 20, (505, 501), True),
+            ("tiled_tall", 9, (701, 699), True)]
+
+
+@pytest.mark.parametrize("kernel,N,n,sources", REPEATED)
+def test_every_shape_repeats_bit_for_bit(kernel, N, n, sources):
+    """As test_runs_repeat_bit_for_bit, for the other shapes."""
+    p = _random_problem(N, n, ("extrapolation", "periodic"), "fp32", 996, 1)
+    s = capi.Stepper.from_problem(p, kernel=kernel, schedule="literal")
+    if sources:
+        for j in range(s.ncomp):
+            X, Y = s.grid_coords(s.moment_info(j)["grid"])
+            s.set_source(j, np.cos(0.7 * j + 3 * X) * np.exp(-Y) / (1 + j % 7))
+    start, ref = s.get_state(), None
+    for _ in range(12):
+        s.set_state(start)
+        s.step(4)
+        got = s.get_state()
+        assert ref is None or got == ref
+        ref = got
+
+
+def test_batch_repeats_bit_for_bit():
+    """The batched pass, strips of tiles of instances of several orders."""
+    probs = [_random_problem(N, n, ("extrapolation", "periodic"), "fp32", 997 + N, 1)
+             for N, n in ((9, (701, 499)), (15, (512, 301)), (3, (1024, 1024)), (12, (333, 640)))]
+    b = capi.Batch.from_problems(probs, kernel="tiled_tall")
+    start, ref = [i.get_state() for i in b.instances], None
+    for _ in range(12):
+        for i, u in zip(b.instances, start):
+            i.set_state(u)
+        b.step(4)
+        b.sync()
+        got = [i.get_state() for i in b.instances]
+        assert ref is None or got == ref
+        ref = got
+    b.close()
