@@ -483,36 +483,35 @@ int odd_pass(starmap_t* h, int which) {
 }
 
 // Boundary copies of the odd grids of state set `set` (0: base, 1: base1).
-template <class T>
 int refresh_odd(starmap_t* h, int set) {
-    GhostPassArgs<T> ga;
+    GhostPassArgs ga;
     const int go[2] = {1, 2};
     for (int q = 0; q < 2; ++q) {
-        ga.g[q] = grid_dev<T>(h, go[q]);
-        if (set) ga.g[q].base = (T*)h->base1[go[q]];
+        ga.g[q] = grid_dev<float>(h, go[q]);
+        if (set) ga.g[q].base = (float*)h->base1[go[q]];
         ga.grid[q] = go[q];
     }
     ga.pitch = h->pitch;
     ga.p[0] = h->p[0];
     ga.p[1] = h->p[1];
-    if (launch_fill_ghosts_pass<T>(ga, h->stream, false)) return cuda_fail(h, cudaGetLastError(), "ghost refresh");
+    if (launch_fill_ghosts_pass(ga, h->stream)) return cuda_fail(h, cudaGetLastError(), "ghost refresh");
     return STARMAP_OK;
 }
 
 // The inner steps of the merged schedule, E_dt O_dt each, as fused launches
 // two at a time (set 0 -> set 1 -> set 0); an odd count runs one unfused.
-template <class T>
+// (FP32: the schedule needs the tiled kernel.)
 int fused_inner_steps(starmap_t* h, long m) {
     int rc;
     if (m % 2) {
-        if ((rc = run_pass<T>(h, false, 1)) || (rc = odd_pass<T>(h, 1))) return rc;
+        if ((rc = run_pass<float>(h, false, 1)) || (rc = odd_pass<float>(h, 1))) return rc;
         --m;
     }
     for (long i = 0; i < m; ++i) {
         const int dir = (int)(i & 1);
         rc = tiled_fused_step(h->tiled, dir, h->stream);
         if (rc) return fail(h, rc, tiled_error(h->tiled));
-        if ((rc = refresh_odd<T>(h, 1 - dir))) return rc;
+        if ((rc = refresh_odd(h, 1 - dir))) return rc;
     }
     return STARMAP_OK;
 }
@@ -525,7 +524,7 @@ int do_steps(starmap_t* h, long n) {
     int rc;
     if (h->cfg.schedule == STARMAP_SCHEDULE_FUSED) {
         if ((rc = odd_pass<T>(h, 0))) return rc;
-        if ((rc = fused_inner_steps<T>(h, n - 1))) return rc;
+        if ((rc = fused_inner_steps(h, n - 1))) return rc;
         if ((rc = run_pass<T>(h, false, 1))) return rc;
         if ((rc = odd_pass<T>(h, 0))) return rc;
     } else if (h->cfg.schedule == STARMAP_SCHEDULE_MERGED) {
@@ -1338,7 +1337,7 @@ int starmap_pass(starmap_t* h, int parity, int which) {
             return fail(h, STARMAP_E_ARG, "parity 2 (a fused pair) needs the fused schedule and which = 1");
         h->have_output = false;
         if (h->ghosts_dirty) { int rc = fill_ghosts_all<float>(h); if (rc) return rc; }
-        return fused_inner_steps<float>(h, 2);
+        return fused_inner_steps(h, 2);
     }
     if ((parity != 0 && parity != 1) || (which != 0 && which != 1)) return fail(h, STARMAP_E_ARG, "parity and which must be 0 or 1");
     h->have_output = false;

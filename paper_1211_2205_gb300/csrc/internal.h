@@ -81,7 +81,7 @@ struct GridDev {
 
 // One output component of the gather pass.
 struct GatherOut {
-    int grid, local, cls, src;
+    int local, cls, src;
     int nxt, nyt;
     int xin[MAXC], yin[MAXC];
 };
@@ -111,10 +111,9 @@ struct GhostArgs {
     int kbegin, kend;             // components to refresh
 };
 
-// Boundary copies of every component of the two output grids of a pass.
-template <class T>
+// Boundary copies of every component of the odd grids (after a fused step).
 struct GhostPassArgs {
-    GridDev<T> g[2];
+    GridDev<float> g[2];
     int grid[2];                  // grid numbers (their x / y type)
     long pitch;
     int p[2];
@@ -131,8 +130,7 @@ struct ReduceArgs {
 // launchers (kernels_gather.cu)
 template <class T> int launch_gather_pass(GatherArgs<T> a, void* stream);
 template <class T> int launch_fill_ghosts(const GhostArgs<T>& a, void* stream);
-// overlap: programmatic dependent launch (after a short tiled pass)
-template <class T> int launch_fill_ghosts_pass(const GhostPassArgs<T>& a, void* stream, bool overlap);
+int launch_fill_ghosts_pass(const GhostPassArgs& a, void* stream);
 template <class T> int launch_reduce(const ReduceArgs<T>& a, double* partials, int nblocks,
                                      double* result, void* stream);
 template <class T> int launch_axpby(T* out, const T* x, const T* y, double alpha, double beta,

@@ -72,43 +72,37 @@ __device__ __forceinline__ void store_sector(float* dst, const float (&v)[8]) {
     reinterpret_cast<float4*>(dst)[0] = make_float4(v[0], v[1], v[2], v[3]);
     reinterpret_cast<float4*>(dst)[1] = make_float4(v[4], v[5], v[6], v[7]);
 }
-__device__ __forceinline__ void store_sector(double* dst, const double (&v)[4]) {
-    reinterpret_cast<double2*>(dst)[0] = make_double2(v[0], v[1]);
-    reinterpret_cast<double2*>(dst)[1] = make_double2(v[2], v[3]);
-}
 
-template <class T>
 __host__ __device__ __forceinline__ int ghost_items(int nx, int ny, bool hx, bool hy) {
     return (hx ? ny : 0) + (hy ? 2 * nx : 0) + 4;
 }
 
-template <class T>
-__device__ __forceinline__ void ghost_item(T* comp, long pitch, int nx, int ny, bool xnode, bool ynode,
+__device__ __forceinline__ void ghost_item(float* comp, long pitch, int nx, int ny, bool xnode, bool ynode,
                                            int px, int py, int i) {
-    constexpr int EPS = 32 / (int)sizeof(T);         // elements per 32-byte sector
+    constexpr int EPS = 32 / (int)sizeof(float);     // elements per 32-byte sector
     const bool hx = px || !xnode, hy = py || !ynode;
     const int xl = px ? nx - 1 : 0, xr = px ? 0 : nx - 1;          // sources of the left / right copies
     const int ylo = py ? ny - 1 : 0, yhi = py ? 0 : ny - 1;        // sources of rows -1 and ny
-    auto at = [&](int x, int y) -> T& { return comp[(long)(y + 1) * pitch + x]; };
+    auto at = [&](int x, int y) -> float& { return comp[(long)(y + 1) * pitch + x]; };
     if (hx) {
         if (i < ny) {
             const int y = i;
-            T* row = &at(0, y);
+            float* row = &at(0, y);
             const int a0 = nx & ~(EPS - 1), b0 = (int)pitch - EPS;
-            T sa[EPS];
+            float sa[EPS];
 #pragma unroll
             for (int e = 0; e < EPS; ++e) {
                 const int x = a0 + e;
-                sa[e] = x < nx ? row[x] : (x == nx ? row[xr] : T(0));
+                sa[e] = x < nx ? row[x] : (x == nx ? row[xr] : 0.f);
             }
             // left copy of row y + 1 (for the last row: the corner (-1, ny))
-            const T left = y + 1 < ny ? at(xl, y + 1) : (hy ? at(xl, yhi) : T(0));
+            const float left = y + 1 < ny ? at(xl, y + 1) : (hy ? at(xl, yhi) : 0.f);
             if (a0 == b0) {
                 sa[EPS - 1] = left;
             } else {
-                T sb[EPS];
+                float sb[EPS];
 #pragma unroll
-                for (int e = 0; e < EPS; ++e) sb[e] = T(0);
+                for (int e = 0; e < EPS; ++e) sb[e] = 0.f;
                 sb[EPS - 1] = left;
                 store_sector(row + b0, sb);
             }
@@ -255,22 +249,18 @@ __global__ void k_fill_ghosts(const GhostArgs<T> A) {
                      (int)(t % 4));
 }
 
-// Boundary copies after a pass whose kernel left them out: blockIdx.y runs
-// over the components of both output grids, threads over the four
-// boundary lines of the component (rows y = 0 and ny - 1, columns x = 0
-// and nx - 1), each point re-stored with its copies (store_point).
-template <class T>
-__global__ void k_fill_ghosts_pass(const GhostPassArgs<T> A) {
-    pdl_trigger();
-    pdl_wait();                         // the pass that wrote these components is done
+// Boundary copies of the odd grids after a fused step, whose kernel leaves
+// them out: blockIdx.y runs over the components of both grids, threads over
+// the items of a component (ghost_item).
+__global__ void k_fill_ghosts_pass(const GhostPassArgs A) {
     const int c = blockIdx.y;
     const int which = c < A.g[0].K ? 0 : 1;
-    const GridDev<T>& G = A.g[which];
+    const GridDev<float>& G = A.g[which];
     const int k = which ? c - A.g[0].K : c;
     const bool xnode = (A.grid[which] & 1) != 0, ynode = (A.grid[which] & 2) != 0;
-    T* comp = G.base + (long)k * G.cstride;
+    float* comp = G.base + (long)k * G.cstride;
     const int nx = G.nx, ny = G.ny;
-    const int items = ghost_items<T>(nx, ny, A.p[0] || !xnode, A.p[1] || !ynode);
+    const int items = ghost_items(nx, ny, A.p[0] || !xnode, A.p[1] || !ynode);
     for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < items; r += gridDim.x * blockDim.x)
         ghost_item(comp, A.pitch, nx, ny, xnode, ynode, A.p[0], A.p[1], r);
 }
@@ -396,14 +386,13 @@ int launch_fill_ghosts(const GhostArgs<T>& a, void* stream) {
     return status_of(cudaGetLastError());
 }
 
-template <class T>
-int launch_fill_ghosts_pass(const GhostPassArgs<T>& a, void* stream, bool overlap) {
+int launch_fill_ghosts_pass(const GhostPassArgs& a, void* stream) {
     const int K = a.g[0].K + a.g[1].K;
     if (K <= 0) return 0;
-    const int len = std::max(ghost_items<T>(a.g[0].nx, a.g[0].ny, true, true), ghost_items<T>(a.g[1].nx, a.g[1].ny, true, true));
+    const int len = std::max(ghost_items(a.g[0].nx, a.g[0].ny, true, true), ghost_items(a.g[1].nx, a.g[1].ny, true, true));
     const dim3 grid((len + 255) / 256, K);
-    const cudaError_t e = launch_pdl(k_fill_ghosts_pass<T>, grid, dim3(256), 0, (cudaStream_t)stream, overlap, a);
-    return status_of(e != cudaSuccess ? e : cudaGetLastError());
+    k_fill_ghosts_pass<<<grid, 256, 0, (cudaStream_t)stream>>>(a);
+    return status_of(cudaGetLastError());
 }
 
 template <class T>
@@ -428,8 +417,6 @@ template int launch_gather_pass<float>(GatherArgs<float>, void*);
 template int launch_gather_pass<double>(GatherArgs<double>, void*);
 template int launch_fill_ghosts<float>(const GhostArgs<float>&, void*);
 template int launch_fill_ghosts<double>(const GhostArgs<double>&, void*);
-template int launch_fill_ghosts_pass<float>(const GhostPassArgs<float>&, void*, bool);
-template int launch_fill_ghosts_pass<double>(const GhostPassArgs<double>&, void*, bool);
 template int launch_reduce<float>(const ReduceArgs<float>&, double*, int, double*, void*);
 template int launch_reduce<double>(const ReduceArgs<double>&, double*, int, double*, void*);
 template int launch_axpby<float>(float*, const float*, const float*, double, double, size_t, void*);

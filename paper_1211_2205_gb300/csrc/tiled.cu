@@ -740,8 +740,7 @@ int tiled_fused_step(TiledPlan* pl, int dir, void* stream) {
 // dependents resident beside them.
 constexpr long long OVERLAP_MAX_STAGES = 1000;
 
-bool tiled_overlap(TiledPlan* pl, bool odd) {
-    if (!pl || !pl->ready) return false;
+static bool tiled_overlap(TiledPlan* pl, bool odd) {
     const int ntiles = pl->tiles_x * pl->tiles_y;
     const int grid = std::max(1, std::min(ntiles, pl->sms * pl->ctas_per_sm));
     return (long long)((ntiles + grid - 1) / grid) * pl->prm[odd ? 1 : 0][0].nstages < OVERLAP_MAX_STAGES;
@@ -812,8 +811,6 @@ void tiled_tile_grid(TiledPlan* pl, int* tx, int* ty) {
 }
 
 int tiled_stage_count(TiledPlan* pl, int P) { return pl ? (int)pl->tab[P].stages.size() : 0; }
-
-int tiled_variant(TiledPlan* pl) { return pl ? pl->variant : 0; }
 
 namespace {
 // One CTA waits, through the passes' own bounded wait, for the phase of an

@@ -40,9 +40,6 @@ int tiled_update(TiledPlan* plan, const SystemMatrices& sys, const std::vector<i
                  const std::vector<char>& frozen, double dx, double dy);
 void tiled_set_coef(TiledPlan* plan, int g, void* coef, int nclasses);
 int tiled_pass(TiledPlan* plan, bool odd, int which, void* stream);
-// Whether the pass is launched with programmatic dependent launch: only for
-// short passes, where the kernel boundary is a visible share of the pass.
-bool tiled_overlap(TiledPlan* plan, bool odd);
 // Temporally fused step: one launch applies the full even update and then
 // the full odd update, tile by tile (fused_kernel.cuh), reading one buffer
 // set and writing the other.  base1: the second set's grid bases (the same
@@ -64,7 +61,6 @@ int tiled_export_params(TiledPlan* plan, void* host4);
 int tiled_smem_bytes(TiledPlan* plan, int P);
 void tiled_tile_grid(TiledPlan* plan, int* tiles_x, int* tiles_y);
 int tiled_stage_count(TiledPlan* plan, int P);
-int tiled_variant(TiledPlan* plan);
 // Self-test of the bounded wait (an mbarrier nothing arrives at); *gave_up = 1
 // when the wait expired and raised the flag as it must.
 int tiled_wait_selftest(int* gave_up);
