@@ -807,15 +807,10 @@ __device__ __forceinline__ void tiled_tiles(const Params& prm, const CUtensorMap
     const int nst = prm.nstages;
     int r = 0, u = 0, issued = 0;
     bool ok = true;
-    // The output warp also has the values that the consumers load one by one
-    // (a source of every target, the decay pairs of every order) brought into
-    // L1, a ring of stages before they are used: such a load stood in the
-    // chain of steps with its whole latency.  150^2 P_39 with both: 168 us per
-    // pass without, 115 with (prefetch.global.L1 instead of the copies: 128;
-    // loads into registers a step or two ahead, in the consumers: 174 to 179).
     // WARM: the output warp also has the values that the consumers load one by
     // one (a source of every target, the decay pairs of every order) brought
-    // into L1, a ring of stages before they are used.
+    // into L1, a ring of stages before they are used: such a load stood in the
+    // chain of steps with its whole latency.
     const uint32_t scratch = base + SCRATCH_OFF;
     // A row of 64 values at any alignment: 9 x 32 bytes, or, for the tiles of ten rows, which leave L1 little
     // room, 3 x 128 (whose other sectors then come from L2).  us per pass, none / 9 / 3: 150^2 P_39 164 / 98 to 103
