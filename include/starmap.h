@@ -91,7 +91,8 @@ extern "C" {
 #define STARMAP_KERNEL_AUTO    0  /* tiled kernel where supported (FP32 2D P_N, N <= 63),
                                      else gather */
 #define STARMAP_KERNEL_GATHER  1  /* one thread per point, CSR loop over moments; FP64 2D P_N: moments
-                                     streamed by order, or one thread per output on small grids */
+                                     streamed by order, or one thread per output on small grids
+                                     and for N <= 2 (the same values bit for bit) */
 #define STARMAP_KERNEL_TILED   2  /* TMA-staged tiles, moments streamed by order (FP32, 2D P_N,
                                      N <= 63); 10-row tiles, but 5-row ones on a grid too
                                      small to give half the SMs a tile and where the tables
