@@ -215,3 +215,24 @@ def test_autotuner_cache_of_other_kernels(tmp_path, monkeypatch):
     assert not b.tuning()[2]
     again = capi.Batch.from_problems(probs, schedule="merged")
     assert again.tuning()[2]
+
+
+@pytest.mark.parametrize("orders,kernel", [((52, 3, 14), "tiled_tall"), ((49, 16, 1), "tiled_tall"),
+                                           ((63, 2, 15), "tiled_short")])
+def test_batch_of_every_tile_shape(orders, kernel):
+    """The shape of a batch's highest order (each weight kept once, two-row
+    bands, 5-row tiles) on instances of low orders too, one of them with a
+    source added to the live batch."""
+    probs = [inputs.Problem(**{**_instance(k, nsteps=3).__dict__, "N": N}) for k, N in enumerate(orders)]
+    b = capi.Batch.from_problems(probs, kernel=kernel)
+    alone = [capi.Stepper.from_problem(p, kernel="tiled", schedule="merged") for p in probs]
+    for s in (b.instances[1], alone[1]):
+        X, _ = s.grid_coords(s.moment_info(1)["grid"])
+        s.set_source(1, np.cos(3 * X))
+    b.step(3)
+    b.sync()
+    for k, s in enumerate(alone):
+        s.step(3)
+        for j in range(s.ncomp):
+            assert np.array_equal(s.moments(j), b.instances[k].moments(j)), (k, j)
+    b.close()
