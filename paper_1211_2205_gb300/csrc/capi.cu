@@ -271,13 +271,14 @@ int rebuild_tables(starmap_t* h) {
 }
 
 // Rows of nx values to device rows of cp.  A 2D copy of pageable memory takes
-// 5 to 7 us longer than a plain one (replacing a source, FP64 and FP32 64^2:
-// 18.8 and 11.5 us, FP32 150^2: 38 and 33), so the copy is plain where it
+// 5 to 7 us longer than a plain one (replacing a source, before the wait of
+// about 4 us below, FP64 and FP32 64^2: 18.8 and 11.5 us, FP32 150^2: 38 and
+// 33), so the copy is plain where it
 // needs no further pass over the values: rows without padding, and FP32, whose
 // conversion writes padded rows as well.  (FP64 padded on the host: 100^2 24 ->
 // 27 us, 1023 x 700 514 -> 863; a narrow FP32 grid would mostly send padding.)
 template <class T>
-cudaError_t upload_rows(void* d, const double* q, int nx, int ny, int cp) {
+cudaError_t upload_rows(void* d, const double* q, int nx, int ny, int cp, cudaStream_t stream) {
     const size_t row = (size_t)nx * sizeof(T), pitch = (size_t)cp * sizeof(T);
     const bool convert = sizeof(T) != sizeof(double);
     std::unique_ptr<T[]> rows;
@@ -294,8 +295,11 @@ cudaError_t upload_rows(void* d, const double* q, int nx, int ny, int cp) {
             }
         from = rows.get();
     }
-    return w == cp ? cudaMemcpy(d, from, pitch * ny, cudaMemcpyHostToDevice)
-                   : cudaMemcpy2D(d, pitch, from, row, row, ny, cudaMemcpyHostToDevice);
+    // on the handle's stream, and waited for: a blocking copy of pageable memory may return before its last part has
+    // landed, and the passes' stream does not wait for the default one
+    const cudaError_t e = w == cp ? cudaMemcpyAsync(d, from, pitch * ny, cudaMemcpyHostToDevice, stream)
+                                  : cudaMemcpy2DAsync(d, pitch, from, row, row, ny, cudaMemcpyHostToDevice, stream);
+    return e == cudaSuccess ? cudaStreamSynchronize(stream) : e;
 }
 
 // Decay coefficients of grid g from the stored material (section 5.5/5.7):
@@ -1037,7 +1041,8 @@ int starmap_set_source(starmap_t* h, int j, const double* q, size_t count) {
     for (size_t i = 0; i < np; ++i) sq += q[i] * q[i];
     h->src_sq[j] = sq;
     const int nx = h->nxg[g], ny = h->nyg[g], cp = h->cpg[g];
-    CK(h->fp32 ? upload_rows<float>(d, q, nx, ny, cp) : upload_rows<double>(d, q, nx, ny, cp), "upload source");
+    CK(h->fp32 ? upload_rows<float>(d, q, nx, ny, cp, h->stream) : upload_rows<double>(d, q, nx, ny, cp, h->stream),
+       "upload source");
     // the pass tables only change when a component gains a source
     return new_slot ? rebuild_tables(h) : STARMAP_OK;
 }
